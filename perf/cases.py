@@ -742,7 +742,7 @@ def _render(case, seed):
             M[..., i, i] = -aI * ds
         for i, j, v in ((0, 1, aQ), (0, 3, aV), (1, 0, aQ), (1, 2, rV), (2, 1, -rV), (2, 3, rQ), (3, 0, aV), (3, 2, -rQ)):
             M[..., i, j] = -v * ds
-        scale = cf[0][ok].max() * 1e20 if bool(ok.any()) else torch.ones((), **f8)
+        scale = cf[0].max() * 1e20 + 1e-200
         for i, v in ((0, cf[0]), (1, cf[1]), (3, cf[2])):
             M[..., i, 4] = v * ds / w ** 3 / scale
         X = torch.zeros_like(M)
