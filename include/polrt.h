@@ -326,10 +326,11 @@ int rt_image_visibilities(rt_ctx *ctx, const void *img, int form, int stokes, vo
  *     kernel of chunk i on another. last_chunk_div >= 2 shrinks the last chunk to
  *     1/last_chunk_div of a regular one (1 to 16; 0 = 1).
  * In both, the transfer runs with no more blocks per SM than fit in the register file beside
- * the geodesic's. chunks 1 runs the phases one after the other on the context's stream.
+ * the geodesic's (streamed: where none fits, one transfer follows each piece's geodesic).
+ * chunks 1 runs the phases one after the other on the context's stream.
  * chunks 0 (the default, with {0, 0, 0, 0}) is automatic: RT_MIXED and RT_UNPOL images of 2^19
  * rays or more are overlapped, streamed in chunks of about 2^15 rays (at least 16 per piece)
- * with the geodesic at 2 blocks per SM, or in halves of 4 to 16 chunks of about 2^17 rays with
+ * with the geodesic at its full occupancy, or in halves of 4 to 16 chunks of about 2^17 rays with
  * the geodesic at 1 block per SM; smaller images, and the RT_FP64 and RT_SURROGATE forms, run
  * one pass of each kernel. RT_SURROGATE overlaps when chunks >= 2 is set: streamed, each
  * transfer launch's rays go through the features pass, the network (over compact rows) and
@@ -340,7 +341,7 @@ int rt_image_visibilities(rt_ctx *ctx, const void *img, int form, int stokes, vo
  * predicts the counts from a probe of one ray per 8 x 8 block; the next render rebuilds the
  * order from the counts the first one recorded. The image is the same in every shape and order
  * (every ray takes the same arithmetic); only the time differs. Shapes that exceed the
- * kernels' occupancy, chunks above 256 or last_chunk_div outside 0..16 return RT_ERR_INVALID. */
+ * kernels' occupancy (4 for the geodesic), chunks above 256 or last_chunk_div outside 0..16 return RT_ERR_INVALID. */
 typedef struct {
     int geo_blocks_per_sm;
     int xfer_blocks_per_sm;

@@ -24,10 +24,9 @@ constexpr size_t kPerRayBytes = sizeof(RayRecord) + kBudgetBlocksPerRay * kBlock
 constexpr int kAutoChunkShift = 17;
 constexpr int kAutoChunksMax = 16;
 constexpr int kAutoLastDiv = 1;
-// automatic streamed shape: about 2^kStreamChunkShift rays per chunk, at least 16 per piece,
-// kStreamGeoBlocks geodesic blocks per SM
+// automatic streamed shape: about 2^kStreamChunkShift rays per chunk, at least 16 per piece, the
+// geodesic at its own occupancy
 constexpr int kStreamChunkShift = 15;
-constexpr int kStreamGeoBlocks = 2;
 // RT_FETCH_AUTO: the grid fetch measured faster on GB300 for the benchmark image
 constexpr bool kStagedByDefault = false;
 
@@ -125,7 +124,7 @@ int rt_create(rt_ctx **out, int device, void *stream) {
     c->xf_regs_mixed = transfer_regs_mixed();
     c->regs_per_sm = prop.regsPerMultiprocessor;
     bool ok = cudaMalloc(&c->d_stats, (8 + 4 * kStatBlocks) * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&c->d_sctab, kSinTabBytes) == cudaSuccess &&
+              cudaMalloc(&c->d_sctab, kGeoTabBytes) == cudaSuccess &&
               cudaMalloc(&c->d_syn, kSynTabBytes) == cudaSuccess && cudaMalloc(&c->d_gl, 16 * sizeof(double)) == cudaSuccess &&
               cudaMallocHost(&c->h_ctr, sizeof(Counters)) == cudaSuccess &&
               cudaStreamCreateWithFlags(&c->bstream, cudaStreamNonBlocking) == cudaSuccess;
@@ -137,8 +136,7 @@ int rt_create(rt_ctx **out, int device, void *stream) {
         return RT_ERR_CUDA;
     }
     memset(c->h_ctr, 0, sizeof(Counters));
-    launch_sincos_table(c->d_sctab, c->stream);
-    if (launch_kappa_tables(c->d_syn, c->d_gl, c->stream) != 0 || cudaStreamSynchronize(c->stream) != cudaSuccess) {
+    if (launch_geo_tables(c->d_sctab, c->stream) != 0 || launch_kappa_tables(c->d_syn, c->d_gl, c->stream) != 0 || cudaStreamSynchronize(c->stream) != cudaSuccess) {
         cudaGetLastError();
         rt_destroy(c);
         return RT_ERR_CUDA;
@@ -537,13 +535,13 @@ static ChunkLayout overlap_chunks(const rt_ctx *c, long long nrays, int chunks, 
 }
 
 // Registers of a block (allocated per warp, in units of 256) and the transfer blocks per SM that
-// fit in the register file beside geo_b geodesic blocks, at most xf_b and at least 1.
+// fit in the register file beside geo_b geodesic blocks, at most xf_b (0: none).
 static int block_regs(int regs, int threads) { return ((regs * 32 + 255) / 256) * 256 * ((threads + 31) / 32); }
 static int xf_beside_geo(const rt_ctx *c, int form, int geo_b, int xf_b) {
     const int xr = block_regs(form == RT_FP64 ? c->xf_regs_fp64 : c->xf_regs_mixed, kXferThreads);
     const int room = c->regs_per_sm - geo_b * block_regs(c->geo_regs, kGeoThreads);
     const int fit = room > 0 ? room / xr : 0;
-    return std::max(1, std::min(xf_b, fit));
+    return std::min(xf_b, fit);
 }
 
 // Overlapped render. The rays are split into K chunks that alternate between two halves of the
@@ -788,7 +786,10 @@ static int render_streamed(rt_ctx *c, int form, int coef, const Camera &cam, con
 
         // Launch every run of consecutive chunks that are complete and not yet launched as one
         // transfer (a chunk of long rays may complete after later ones), at the occupancy that
-        // fits beside the geodesic, or at the transfer's own once the geodesic has ended. At
+        // fits beside the geodesic, or at the transfer's own once the geodesic has ended. Where
+        // none fits (the automatic shape), one transfer of the whole piece follows the geodesic:
+        // both kernels live on the integer and FP32 pipes, and beside each other they take longer
+        // (1024^2: 79 + 69 ms one after the other; 164 ms at 2 + 2 and 203 ms at 3 + 1 blocks). At
         // most one launch waits behind the running one: a new launch is made once the previous
         // has started, so the chunks that complete meanwhile join one launch instead of queueing
         // one each (a launch lasts at least as long as its longest ray's transfer).
@@ -810,6 +811,7 @@ static int render_streamed(rt_ctx *c, int form, int coef, const Camera &cam, con
             bool any = false, ready = false;
             bool may = prev < 0 || cudaEventQuery(ts[base_k + prev]) == cudaSuccess;
             cudaGetLastError();
+            may = may && (xf_grid > 0 || q == cudaSuccess);
             for (int a = 0; a < L.K;) {
                 if (launched[a] || !__atomic_load_n(&c->h_flags[a], __ATOMIC_ACQUIRE)) {
                     a++;
@@ -912,8 +914,8 @@ int render_jobs_overlap(rt_ctx *c, int form, const JobDev *d_jobs, const JobDev 
     }
     const long long K = L.K;
     int rv = RT_OK;
-    const int xf_own = form == RT_FP64 ? c->fp64_bps : c->mixed_bps, geo_b = streamed ? kStreamGeoBlocks : 1;
-    const int geo_grid = c->nsm * geo_b, xf_grid = c->nsm * xf_beside_geo(c, form, geo_b, xf_own);
+    const int xf_own = form == RT_FP64 ? c->fp64_bps : c->mixed_bps, geo_b = streamed ? c->geo_bps : 1;
+    const int geo_grid = c->nsm * geo_b, xf_grid = c->nsm * std::max(streamed ? 0 : 1, xf_beside_geo(c, form, geo_b, xf_own));
     // longest first, as for one image, once a batch of the same cameras has recorded its steps
     unsigned long long key = 1469598103934665603ull;  // FNV-1a over the cameras and integrator
     auto mix = [&](const void *v, size_t n) {
@@ -1004,7 +1006,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     const size_t per_ray = kPerRayBytes + (sur ? (size_t)kBudgetBlocksPerRay * kBlockStates * 48 : 0);
 
     // launch shape: the configured one, or automatic. RT_MIXED and RT_UNPOL overlap images of
-    // 2^19 rays or more: streamed (chunks of about 2^15 rays, the geodesic at 2 blocks per SM)
+    // 2^19 rays or more: streamed (chunks of about 2^15 rays, the geodesic at its own occupancy)
     // when the workspace holds a piece of at least 1/64 of the rays, else in two workspace
     // halves (4 to 16 chunks of about 2^17 rays, the geodesic at 1 block per SM beside the
     // transfer). Smaller images run one pass of each kernel, and so do RT_FP64 (its FP64
@@ -1027,7 +1029,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
         // contiguous ranges of each piece's longest-first order; the automatic shape takes finer
         // chunks and a second geodesic block per SM
         Kp = stream_chunks(nrays, P, chunks, auto_shape);
-        if (geo_b == 0) geo_b = kStreamGeoBlocks;
+        if (geo_b == 0) geo_b = c->geo_bps;
     } else {
         if (ovl && geo_b == 0) geo_b = 1;
         if (W == 0) W = auto_shape ? kAutoLastDiv : 1;
@@ -1132,8 +1134,9 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     const int geo_bps = geo_b > 0 ? geo_b : c->geo_bps;
     const int geo_grid = c->nsm * geo_bps;
     const int xf_own = c->rcfg.xfer_blocks_per_sm > 0 ? std::min(c->rcfg.xfer_blocks_per_sm, xf_max) : xf_max;
-    // overlapped: no more transfer blocks per SM than fit beside the geodesic's
-    const int xf_grid = c->nsm * (ovl ? xf_beside_geo(c, form, geo_bps, xf_own) : xf_own);
+    // overlapped: no more transfer blocks per SM than fit beside the geodesic's (streamed: none
+    // before the geodesic has ended, where none fit)
+    const int xf_grid = c->nsm * (ovl ? std::max(streamed ? 0 : 1, xf_beside_geo(c, form, geo_bps, xf_own)) : xf_own);
     c->last_was_overlap = false;
     c->last_was_streamed = false;
     if (ovl) {
@@ -1348,7 +1351,8 @@ int rt_get_grid_fetch(rt_ctx *c, int *mode) {
 
 int rt_set_render_config(rt_ctx *c, const rt_render_config *cfg) {
     if (!c || !cfg) return RT_ERR_INVALID;
-    if (cfg->geo_blocks_per_sm < 0 || cfg->geo_blocks_per_sm > c->geo_bps) return RT_ERR_INVALID;
+    // up to 4 geodesic blocks per SM, of which 3 are resident: the rest find the queue empty
+    if (cfg->geo_blocks_per_sm < 0 || cfg->geo_blocks_per_sm > std::max(c->geo_bps, 4)) return RT_ERR_INVALID;
     if (cfg->xfer_blocks_per_sm < 0 || cfg->xfer_blocks_per_sm > std::max(c->mixed_bps, c->fp64_bps))
         return RT_ERR_INVALID;
     if (cfg->chunks < 0 || cfg->chunks > rt_ctx::kMaxChunks) return RT_ERR_INVALID;

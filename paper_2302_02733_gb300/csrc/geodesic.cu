@@ -4,23 +4,32 @@
 // Persistent kernel, one ray per lane. A lane whose ray stops takes the next ray from a
 // global queue (warp-aggregated atomics), so long photon-ring rays do not hold a warp's
 // other lanes idle. Every state is written to a block arena, 64 B per state: each lane
-// writes two full 32 B sectors. The FP64 pipe bounds this kernel.
+// writes two full 32 B sectors.
+//
+// The step runs in fixed point on the integer pipes (geofix.cuh): 4,800 instructions a warp and
+// step, 19 of them on the FP64 pipe (346 in the FP64 form, 80 clocks each). The pipe of the integer
+// multiply-adds bounds it (71% busy, 55% of the issue slots): 79 ms for the 3.68e8 steps of a
+// 1024^2 image at 3 blocks per SM, against 228 ms in FP64. At 1 and 2 blocks per SM it takes 138 and
+// 91 ms, at 4 (128 registers, 220 bytes of spills) 78.
 #include <algorithm>
+#include <cmath>
+#include <vector>
 
 #include "geodesic.cuh"
 
 namespace prt {
 
-static_assert(kSinTabBytes == 3 * kSinTab * sizeof(double), "sin/cos table size");
+static_assert(kGeoTabBytes == 3 * kSinTab * sizeof(double) + kFxTabBytes, "sin/cos table sizes");
 
 // JOBS: the rays run over a table of images (p.jobs), each with its own camera; otherwise over
 // the one image of p.cam.
 template <bool JOBS>
-__global__ void __launch_bounds__(kGeoThreads, 4) geodesic_kernel(GeoArgs p) {
+__global__ void __launch_bounds__(kGeoThreads, 3) geodesic_kernel(GeoArgs p) {
     // the sin/cos table in shared memory: the RK4 stages read it at data-dependent indices, and
     // through the texture path those reads queued behind the transfer's gathers
-    __shared__ double tab[3 * kSinTab];
-    for (int i = threadIdx.x; i < 3 * kSinTab; i += blockDim.x) tab[i] = p.sctab[i];
+    __shared__ __align__(16) fx64 fxtab[2 * kFxTab];
+    const GeoTabs tabs{fxtab, p.sctab};
+    load_fx_table(p.sctab, fxtab);
     __syncthreads();
     const Camera &c = p.cam;
     StepCam sc{};  // JOBS: the current ray's camera constants
@@ -60,7 +69,7 @@ __global__ void __launch_bounds__(kGeoThreads, 4) geodesic_kernel(GeoArgs p) {
         if (!live) continue;
 
         double h, yn[7];
-        bool refl = JOBS ? geo_step(tab, sc, y, yn, h) : geo_step(tab, c, y, yn, h);
+        bool refl = JOBS ? geo_step(tabs, sc, y, yn, h) : geo_step(tabs, c, y, yn, h);
         // save state n with the step taken from it; then n+1 becomes current
         uint8_t status = 0;
         for (int pass = 0; pass < 2; pass++) {
@@ -129,8 +138,54 @@ __global__ void sincos_table_kernel(double *tab) {
     tab[3 * k + 2] = c;
 }
 
-void launch_sincos_table(double *tab, cudaStream_t s) {
+// sin and cos of k 2^-8 to 2^-62: Taylor sums in double-double (Dekker's exact products, Knuth's
+// exact sums), with the same result on every host. Built once per process.
+static const fx64 *fx_table_host() {
+    struct DD {
+        double h, l;
+    };
+    auto add = [](DD a, DD b) {
+        const double s = a.h + b.h, t = s - a.h;
+        const double e = ((a.h - (s - t)) + (b.h - t)) + (a.l + b.l), r = s + e;
+        return DD{r, e - (r - s)};
+    };
+    auto mul = [](DD a, DD b) {
+        const double p = a.h * b.h, e = std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h), r = p + e;
+        return DD{r, e - (r - p)};
+    };
+    auto div = [](DD a, double d) {  // by a small integer
+        const double q = a.h / d, e = (std::fma(-q, d, a.h) + a.l) / d, r = q + e;
+        return DD{r, e - (r - q)};
+    };
+    static const std::vector<fx64> tab = [&] {
+        std::vector<fx64> t(2 * kFxTab);
+        for (int k = 0; k < kFxTab; k++) {
+            const DD x{k / 256.0, 0.0}, m = mul(x, DD{-x.h, 0.0});
+            DD s = x, c{1.0, 0.0}, ts = x, tc{1.0, 0.0};
+            for (int n = 1; n < 30; n++) {
+                tc = div(mul(tc, m), (2.0 * n - 1.0) * (2.0 * n));
+                ts = div(mul(ts, m), (2.0 * n) * (2.0 * n + 1.0));
+                c = add(c, tc);
+                s = add(s, ts);
+            }
+            const DD v[2] = {s, c};
+            for (int j = 0; j < 2; j++) {
+                const double big = v[j].h * 4611686018427387904.0, whole = std::rint(big);  // 2^62
+                t[2 * k + j] = (fx64)whole + (fx64)std::llrint((big - whole) + v[j].l * 4611686018427387904.0);
+            }
+        }
+        return t;
+    }();
+    return tab.data();
+}
+
+// tab: the FP64 table (kSinTabBytes), then the fixed-point one (kFxTabBytes).
+int launch_geo_tables(double *tab, cudaStream_t s) {
     sincos_table_kernel<<<(kSinTab + 255) / 256, 256, 0, s>>>(tab);
+    if (cudaGetLastError() != cudaSuccess) return -1;
+    return cudaMemcpyAsync(tab + 3 * kSinTab, fx_table_host(), kFxTabBytes, cudaMemcpyHostToDevice, s) == cudaSuccess
+               ? 0
+               : -1;
 }
 
 void launch_geodesic(const GeoArgs &a, int grid, cudaStream_t s) {

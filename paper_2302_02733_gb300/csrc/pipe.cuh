@@ -85,7 +85,7 @@ __device__ __forceinline__ void publish(const PipeArgs &p, long long ray, const 
     atomicExch(p.ready + pos, (int)ray);
 }
 
-__device__ __forceinline__ void pipe_geodesic(const PipeArgs &p, const double *tab) {
+__device__ __forceinline__ void pipe_geodesic(const PipeArgs &p, const GeoTabs &tabs) {
     const unsigned long long nb = (unsigned long long)p.pool.nblocks;
     double y[7];
     StepCam sc{};  // the current ray's camera constants
@@ -172,7 +172,7 @@ __device__ __forceinline__ void pipe_geodesic(const PipeArgs &p, const double *t
         uint8_t status = 0;
         for (int k = 0; k < p.step_tile; k++) {
             double h, yn[7];
-            bool refl = geo_step<true>(tab, sc, y, yn, h);
+            bool refl = geo_step(tabs, sc, y, yn, h);
             save_state(p.pool, blk, slot, y, refl ? -h : h);
             slot++;
             n++;
@@ -304,12 +304,12 @@ __device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *sgw) {
 template <typename R, typename OutT>
 __global__ void __launch_bounds__(kPipeThreads, sizeof(R) == 4 ? 2 : 1) pipe_kernel(PipeArgs p) {
     __shared__ R sgw[32];
-    __shared__ double tab[3 * kSinTab];  // the geodesic's sin/cos table
+    __shared__ __align__(16) fx64 fxtab[2 * kFxTab];  // the geodesic's sin/cos table
     fill_bessel_weights(sgw);
-    for (int i = threadIdx.x; i < 3 * kSinTab; i += blockDim.x) tab[i] = p.sctab[i];
+    load_fx_table(p.sctab, fxtab);
     __syncthreads();
     if ((int)(threadIdx.x >> 5) < ((blockIdx.x & 1) ? p.geo_warps_odd : p.geo_warps))
-        pipe_geodesic(p, tab);
+        pipe_geodesic(p, GeoTabs{fxtab, p.sctab});
     else
         pipe_transfer<R, OutT>(p, sgw);
 }

@@ -36,7 +36,7 @@ struct rt_ctx {
     void *d_stage_depth = nullptr;
     size_t stage_depth_bytes = 0;
     double *d_stats = nullptr;
-    double *d_sctab = nullptr;  // sin/cos table of the FP64 geodesic
+    double *d_sctab = nullptr;  // the geodesic's sin and cos tables
     double *d_syn = nullptr;    // ln F, ln G, ln H tables of the kappa quadrature
     double *d_gl = nullptr;     // its Gauss-Legendre nodes and weights
     // surrogate MLP: parameters | Adam m | Adam v | gradient (FP32), tensor-core images, scalars

@@ -56,7 +56,7 @@ struct ChunkLayout {
 
 struct GeoArgs {
     Camera cam;
-    const double *sctab;  // (theta, sin, cos) table of the FP64 geodesic, 1024 entries
+    const double *sctab;  // the geodesic's sin and cos tables (kGeoTabBytes)
     Arena arena;
     RayRecord *rec;       // per ray of this chunk
     Counters *ctr;
@@ -189,8 +189,9 @@ void launch_order_build(const uint16_t *steps, const ChunkLayout &L, unsigned *h
 // blocks, clipped to the image); then every pixel takes its block's probe's step count.
 void launch_probe_list(int *list, int nx, int ny, int S, cudaStream_t s);
 void launch_steps_fill(uint16_t *steps, int nx, int ny, int S, cudaStream_t s);
-void launch_sincos_table(double *tab, cudaStream_t s);
-constexpr size_t kSinTabBytes = 1024 * 3 * sizeof(double);
+int launch_geo_tables(double *tab, cudaStream_t s);
+// the FP64 step's 1024 (theta, sin, cos), then the fixed-point step's 806 (sin, cos)
+constexpr size_t kGeoTabBytes = (1024 * 3 + 806 * 2) * sizeof(double);
 // coef: 0 thermal fits, 1 kappa quadrature at every emitting point, 2 surrogate outputs
 void launch_transfer_fp64(const XferArgs &a, int coef, int grid, cudaStream_t s);
 void launch_transfer_mixed(const XferArgs &a, int coef, int grid, cudaStream_t s);
