@@ -6,14 +6,16 @@
 // several times faster here than on the FP64 pipe, and carries more bits: the null momentum's
 // components share one scale, which bounds every term, so no product or sum needs an exponent of
 // its own. Against the same step in extended precision the new r, theta and phi are 30% closer than
-// the FP64 form's and the momentum as close (their FP64 rounding dominates).
+// the FP64 form's and the momentum as close (its FP64 rounding dominates); whole rays end 20 to 30%
+// closer to those traced in quadruple precision.
 //
 // Scaling, once per step. rho = 2^e with r / rho in [1/2, 1); x = r / rho, alpha = a / rho. The
 // momentum is taken as W, R = K^r, v = rho K^theta and u = rho sin(theta) K^phi, divided by a
 // 2^kap that puts the largest below 1/4 (the physical components of a null vector, so all are
-// bounded by the same number and an absolute error of 2^-60 of it is far below the rounding of
-// the FP64 angles). K^phi alone grows as 1 / sin(theta) toward the axis: P = rho K^phi 2^-kap
-// 2^-z, u = s P 2^z. The affine step becomes hh = h 2^kap / rho, and every rate is dimensionless.
+// bounded by the same number). Far from the hole v, u and the spin are small beside W and R, and
+// an absolute error in v or u moves the ray's impact parameter by r times that: so they are kept 2^g
+// times larger (g <= e - 1, which keeps |alpha| 2^g below 1/2). K^phi alone grows as 1 / sin(theta) toward the axis: P = rho K^phi 2^-kap
+// 2^-z, u = s P 2^z (P, v and u times 2^g). The affine step becomes hh = h 2^kap / rho, and every rate is dimensionless.
 //
 // Fx<Q> is a signed 64-bit integer m standing for m 2^-Q. A product of Fx<A> and Fx<B> is
 // Fx<A + B - 64>; sums need equal Q. The bound of each quantity is written beside it, with
@@ -219,8 +221,8 @@ __device__ __forceinline__ Fx<Q> fx_recip(Fx<60> v) {
 
 // The step's scale: exponents and spin.
 struct FxScale {
-    int e, kap, z;
-    Fx<63> al;        // a / rho, |al| < 1/2
+    int e, kap, g, z;
+    Fx<63> al;        // a 2^g / rho, |al| < 1/2
     Fx<64> nal2;      // minus its square, > -1/4
     unsigned klim, plim;  // bounds of the rates: hh |rate| < 1/4, below 2 (Q60) and 8 (P's, Q58), in units of 2^32
 };
@@ -251,15 +253,17 @@ __device__ __forceinline__ unsigned fx_beyond(fx64 m, fx64 lo, fx64 hi) {
 //   F_ph = 2 r K^r s^2 K^ph + 2 (r^2 + a^2) s c K^th K^ph - 2 a s c K^th T - a s^2 F_t,
 //   F_th = 2 r K^r K^th - a^2 s c K^th^2 - (r^2 + a^2) s c K^ph^2 + 2 a s c K^ph T - V^2 dq/dth / 2.
 // In units of rho and 2^kap, with n for "minus":
-//   isig = rho^2 / Sigma, qh = q rho / 2, Dr = (rho^2 / 2) dq/dr, Dt = (rho / 4) dq/dth,
-//   del = (rho^2 / 2) Dq, At = (rho^2 / 2) F_t, At2 = rho F_t, Fr = rho F_r, Fm = Fr - At2,
-//   Ap = F_ph = s J + 2 sa c v u, F_th = F1 - sa c u P 2^z.
+//   isig = rho^2 / Sigma, qh = q rho / 2, Dr = (rho^2 / 2) dq/dr, del = (rho^2 / 2) Dq,
+//   At = (rho^2 / 2) F_t, At2 = rho F_t, Fr = rho F_r, Fm = Fr - At2;
+// and, in units of 2^-g for each factor of v, u, P or alpha,
+//   Dt = (rho / 4) dq/dth 2^2g, Ap = F_ph 2^g = s J + 2 sa c v u 2^-g, F_th 2^g = F1 - sa c u P 2^(z - g).
 // Every term in 1 / sin is written with P. A negative number in bad is a bound that failed.
 __device__ __forceinline__ void fx_rates(const FxScale &S, const FxState &y, Fx<62> s, Fx<62> c, fx64 nk[4], unsigned &bad) {
-    const int e1 = S.e - 1;
+    const int e1 = S.e - 1, g = S.g, g2 = 2 * S.g, g3 = 3 * S.g;
     // position terms
-    const Fx<60> na2s2 = S.nal2 * (s * s);                            // >= -1/4
-    const Fx<60> sa = y.x * y.x - S.nal2.dn<4>();                     // <= 1.46
+    const Fx<64> nal2 = S.nal2.over(g2);
+    const Fx<60> na2s2 = nal2 * (s * s);                              // >= -1/4
+    const Fx<60> sa = y.x * y.x - nal2.dn<4>();                       // <= 1.46
     const Fx<60> isig = fx_recip(sa + na2s2);                         // <= 4.94
     const Fx<61> qh = (y.x * isig).up<3>();                           // <= 2.23
     const Fx<61> q = qh.over(e1);
@@ -273,35 +277,37 @@ __device__ __forceinline__ void fx_rates(const FxScale &S, const FxState &y, Fx<
     // contractions with the momentum
     const Fx<63> u{fx_shl((s * y.P).m, S.z + 2)};
     const Fx<64> au = (S.al * u).up<2>();                             // 0.16
-    const Fx<62> V = y.W.dn<1>() - s * au;                            // 0.47
+    const Fx<62> V = y.W.dn<1>() - s * au.over(g2);                   // 0.47
     const Fx<60> V2 = V * V;                                          // 0.22
     const Fx<64> V2e{fx_shl(V2.m, 3) >> e1};                          // V^2 / rho
     const Fx<63> cv = (c * y.v).up<2>(), cu = (c * u).up<2>();
-    const Fx<62> E2{(cv * au).m};                                     // 2 cv au
+    const Fx<62> E2{(cv * au).m >> g3};                               // 2 a s c K^th K^ph rho
     const Fx<62> v2 = y.v * y.v, uv2 = fx_dot(u, u, y.v, y.v);        // 0.2
-    const Fx<61> ndel = fx_dot(y.R, nDr, y.v, nDt.dn<1>().twice()).up<2>();  // 2.4
+    const Fx<61> ndel = fx_dot(y.R, nDr, y.v, nDt.dn<1>().twice().over(g3)).up<2>();  // 2.4
     const Fx<59> nAt = fx_dot(ndel, V, qh, E2);                       // 1.4
     const Fx<60> nAt2{fx_shl(nAt.m, 1) >> e1};
-    const Fx<61> nFm = E2.dn<1>() + fx_dot(y.x, uv2, -nDr, V2e).up<1>();  // 0.85
+    const Fx<61> nFm = E2.dn<1>() + fx_dot(y.x, uv2.over(g2), -nDr, V2e).up<1>();  // 0.85
     const Fx<61> nFr = nAt2.up<1>() + nFm;                            // 2.2
     const Fx<62> T = y.R.dn<1>() + (q * V).up<3>();                   // 1.4
     const Fx<63> xR = (y.x * y.R).up<2>();                            // 0.35
-    const Fx<61> G = fx_dot(xR, u, S.al, -((cv * T).up<2>())).twice();  // 0.65
-    const Fx<62> scv = (sa * cv).up<3>();                             // 0.46
+    const Fx<61> G = fx_dot(xR, u, S.al, -((cv * T).up<2>().over(g))).twice();  // 0.65
+    const Fx<62> scv = (sa * cv).up<3>().over(g);                     // 0.46
     const Fx<61> J = G + as * nAt2.up<2>();                           // 1.4
     const Fx<60> Ap = fx_dot(s, J.up<1>(), scv.twice(), u);           // 1.7
     // W and R: g^tt = -(1 + q), g^tr = q, g^rr = Delta / Sigma, g^rph = a / Sigma;
     // (r^2 + a^2) / Sigma = 1 + a^2 s^2 / Sigma
-    const Fx<60> Y = fx_dot_fine(nA.up<3>(), nFr, ai, Ap.up<2>()) - nFr.dn<1>();
+    const Fx<60> Y = fx_dot_fine(nA.up<3>(), nFr, ai, Ap.up<2>().over(g2)) - nFr.dn<1>();
     const Fx<60> nkW = nAt2 + Y, nkR = q * nFm.up<2>() + Y;
     // theta
     const Fx<64> acu = (S.al * cu).up<2>();                           // 0.16
-    const Fx<61> F1 = fx_dot(xR.twice(), y.v, acu.twice(), T) + fx_dot(nasc.dn<1>(), v2, nDt.twice(), V2e);  // 0.9
+    const Fx<61> F1 = fx_dot(xR.twice(), y.v, acu.twice().over(g), T) +
+                      fx_dot(nasc.dn<1>(), v2.over(g3), nDt.twice().over(g), V2e);  // 0.9
     const fx64 cuP = (cu * y.P).m >> 2;                               // Q60
-    const Fx<63> cz{fx_shl(cuP, S.z + 3)};                            // c u^2 / s, < 1
+    const int zg = S.z - g, zl = zg > 0 ? zg : 0;
+    const Fx<63> cz{fx_shl(cuP >> (zl - zg), zl + 3)};                // c u^2 / s, < 1
     const Fx<60> npi{fx_shl(nA.m, 1) - (1ll << 60)};                  // -(r^2 + a^2) / Sigma
     const Fx<60> nkv = fx_dot_fine(isig, F1.up<2>(), npi, cz);
-    // phi: (isig / s) (2 sa c v P + (al s Fm + G) / 2^z)
+    // phi: (isig / s) (2 sa c v P 2^-g + (al s Fm + G) / 2^z)
     const fx64 sm = s.m < (1ll << 62) ? s.m : (1ll << 62) - 1;
     const int zs = fx_clz((unsigned long long)(sm | 1)) - 2;          // s 2^zs in [1/2, 1)
     const Fx<61> isn = fx_recip<61>(Fx<60>{fx_shl(sm, zs) >> 2});
@@ -316,7 +322,7 @@ __device__ __forceinline__ void fx_rates(const FxScale &S, const FxState &y, Fx<
            fx_outside(y.P.m, 0x28000000u) | fx_outside(u.m, 0x28000000u);
     bad |= fx_beyond(y.x.m, 2075258708292324556ll, 5072854620270126694ll);  // 0.45, 1.1
     bad |= fx_beyond(s.m, 1ll << 52, (1ll << 62) + (1ll << 40));
-    bad |= fx_outside(cuP, 1u << (28 - S.z)) | fx_outside(B.m, 3u << 26) | fx_outside(nA.m, 1u << 27);
+    bad |= fx_outside(cuP, 1u << (28 - zl)) | fx_outside(B.m, 3u << 26) | fx_outside(nA.m, 1u << 27);
     bad |= fx_outside(nkW.m, S.klim) | fx_outside(nkR.m, S.klim) | fx_outside(nkv.m, S.klim) | fx_outside(nkP.m, S.plim >> zs);
 }
 
@@ -332,8 +338,6 @@ __device__ __forceinline__ bool fx_step(const fx64 *__restrict__ tab, double a, 
     FxState b, t;
     b.x.m = fx_from(y[0], 62 - S.e);
     b.th.m = fx_from(y[1], 61);
-    S.al.m = fx_from(a, 63 - S.e);
-    S.nal2 = -((S.al * S.al).up<2>());
     t = b;
     int hx = 0;
     Fx<62> hm{0};  // hh = hm 2^hx with hm in [1/2, 1)
@@ -346,14 +350,18 @@ __device__ __forceinline__ bool fx_step(const fx64 *__restrict__ tab, double a, 
         Fx<62> s, c;
         fx_sincos(tab, t.th, s, c);
         if (st == 0) {
-            // momentum: the largest of |W|, |R|, rho |K^theta|, rho sin |K^phi| below 2^(kap - 2)
+            // the largest of |W|, |R|, rho |K^theta|, rho sin |K^phi| below 2^(kap - 2), and the
+            // last two below 2^(kap - g - 2)
             const int ep = ex(y[6]) + S.e;
             const int x1 = ex(y[4]), x2 = ex(y[5]) + S.e, x3 = ep + 2 - fx_clz((unsigned long long)(s.m | 1));
+            const int xt = x2 > x3 ? x2 : x3;
             int kap = ex(y[3]);
             kap = kap > x1 ? kap : x1;
-            kap = kap > x2 ? kap : x2;
-            kap = (kap > x3 ? kap : x3) + 2;
-            S.z = ep + 2 - kap;
+            kap = (kap > xt ? kap : xt) + 2;
+            S.g = kap - 2 - xt;
+            S.g = S.g < S.e - 1 ? S.g : S.e - 1;
+            const int kt = kap - S.g;
+            S.z = ep + 2 - kt;
             S.z = S.z < 0 ? 0 : S.z;
             hx = hx0 + kap - S.e;
             bad |= (unsigned)(200 - kap) | (unsigned)(kap + 200) | (unsigned)(11 - S.z) | (unsigned)(3 - hx) |
@@ -364,8 +372,10 @@ __device__ __forceinline__ bool fx_step(const fx64 *__restrict__ tab, double a, 
             S.plim = 1u << (24 - (hx < -5 ? -5 : hx));
             b.W.m = fx_from(y[3], 63 - kap);
             b.R.m = fx_from(y[4], 63 - kap);
-            b.v.m = fx_from(y[5], 63 - kap + S.e);
-            b.P.m = fx_from(y[6], 63 - kap - S.z + S.e);
+            b.v.m = fx_from(y[5], 63 - kt + S.e);
+            b.P.m = fx_from(y[6], 63 - kt - S.z + S.e);
+            S.al.m = fx_from(a, 63 - S.e + S.g);
+            S.nal2 = -((S.al * S.al).up<2>());
             t = b;
             hm.m = fx_from(h, 62 - hx0);
         }
@@ -389,7 +399,7 @@ __device__ __forceinline__ bool fx_step(const fx64 *__restrict__ tab, double a, 
         // the next stage: positions advance with this stage's momentum
         const int hs = st < 2 ? hx - 1 : hx;
         t.x.m = b.x.m + scaled(fx_mulhi(hm.m, t.R.m), hs + 1);
-        t.th.m = b.th.m + scaled(fx_mulhi(hm.m, t.v.m), hs);
+        t.th.m = b.th.m + scaled(fx_mulhi(hm.m, t.v.m), hs - S.g);
         t.W.m = b.W.m - scaled(fx_mulhi(hm.m, nk[0]), hs + 5);
         t.R.m = b.R.m - scaled(fx_mulhi(hm.m, nk[1]), hs + 5);
         t.v.m = b.v.m - scaled(fx_mulhi(hm.m, nk[2]), hs + 5);
@@ -401,12 +411,12 @@ __device__ __forceinline__ bool fx_step(const fx64 *__restrict__ tab, double a, 
     const Fx<65> sixth{6148914691236517205ll};
     const Fx<64> h6 = (hm * sixth).up<1>();
     out[0] = y[0] + fx_to(fx_mulhi(hm.m, b.R.m - scaled(fx_mulhi(h6.m, SP[0]), hx + 4)), 61 - hx - S.e);
-    out[1] = y[1] + fx_to(fx_mulhi(hm.m, b.v.m - scaled(fx_mulhi(h6.m, SP[1]), hx + 4)), 61 - hx);
-    out[2] = y[2] + fx_to(fx_mulhi(hm.m, b.P.m - scaled(fx_mulhi(h6.m, SP[2]), hx + 6)), 61 - hx - S.z);
+    out[1] = y[1] + fx_to(fx_mulhi(hm.m, b.v.m - scaled(fx_mulhi(h6.m, SP[1]), hx + 4)), 61 - hx + S.g);
+    out[2] = y[2] + fx_to(fx_mulhi(hm.m, b.P.m - scaled(fx_mulhi(h6.m, SP[2]), hx + 6)), 61 - hx - S.z + S.g);
     out[3] = y[3] - fx_to(fx_mulfine<2>(h6.m, SK[0]), 61 - hx - S.kap);
     out[4] = y[4] - fx_to(fx_mulfine<2>(h6.m, SK[1]), 61 - hx - S.kap);
-    out[5] = y[5] - fx_to(fx_mulfine<2>(h6.m, SK[2]), 61 - hx - S.kap + S.e);
-    out[6] = y[6] - fx_to(fx_mulfine<2>(h6.m, SK[3]), 59 - hx - S.kap - S.z + S.e);
+    out[5] = y[5] - fx_to(fx_mulfine<2>(h6.m, SK[2]), 61 - hx - S.kap + S.g + S.e);
+    out[6] = y[6] - fx_to(fx_mulfine<2>(h6.m, SK[3]), 59 - hx - S.kap - S.z + S.g + S.e);
     return true;
 }
 
