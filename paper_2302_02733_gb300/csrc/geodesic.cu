@@ -190,6 +190,7 @@ int launch_geo_tables(double *tab, cudaStream_t s) {
 }
 
 void launch_geodesic(const GeoArgs &a, int grid, cudaStream_t s) {
+    grid = ray_grid(grid, a.nrays, kGeoThreads);
     if (a.jobs)
         geodesic_kernel<true><<<grid, kGeoThreads, 0, s>>>(a);
     else

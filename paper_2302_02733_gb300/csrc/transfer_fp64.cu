@@ -3,6 +3,7 @@
 
 namespace prt {
 void launch_transfer_fp64(const XferArgs &a, int coef, int grid, cudaStream_t s) {
+    grid = ray_grid(grid, a.nrays, kXferThreads);
     switch (coef) {
         case 0:
             if (a.jobs)

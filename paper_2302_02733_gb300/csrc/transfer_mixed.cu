@@ -6,6 +6,7 @@
 
 namespace prt {
 void launch_transfer_mixed(const XferArgs &a, int coef, int grid, cudaStream_t s) {
+    grid = ray_grid(grid, a.nrays, kXferThreads);
     switch (coef) {
         case 0:
             if (a.jobs)
@@ -19,6 +20,7 @@ void launch_transfer_mixed(const XferArgs &a, int coef, int grid, cudaStream_t s
     }
 }
 void launch_transfer_staged(const XferArgs &a, const CUtensorMap &map, int grid, cudaStream_t s) {
+    grid = ray_grid(grid, a.nrays, kXferThreads);
     transfer_kernel_staged<0><<<grid, kXferThreads, 0, s>>>(a, map);
 }
 int transfer_blocks_per_sm_staged() {
@@ -27,12 +29,14 @@ int transfer_blocks_per_sm_staged() {
     return n > 0 ? n : 1;
 }
 void launch_unpol(const XferArgs &a, int grid, cudaStream_t s) {
+    grid = ray_grid(grid, a.nrays, kXferThreads);
     if (a.jobs)
         unpol_kernel<float, true><<<grid, kXferThreads, 0, s>>>(a);
     else
         unpol_kernel<float><<<grid, kXferThreads, 0, s>>>(a);
 }
 void launch_sur_features(const XferArgs &a, int grid, cudaStream_t s) {
+    grid = ray_grid(grid, a.nrays, kXferThreads);
     sur_features_pass<float><<<grid, kXferThreads, 0, s>>>(a);
 }
 static int func_regs(const void *f) {
