@@ -335,6 +335,10 @@ int rt_set_workspace(rt_ctx *c, void *dev_ptr, size_t bytes) {
 constexpr size_t kSurBlockBytes = (size_t)kBlockStates * (16 + 32 + 4);
 constexpr size_t kSurPerRayBytes = kPerRayBytes + (size_t)kBudgetBlocksPerRay * kSurBlockBytes;
 
+// Bytes per arena block the FP64 form's one-pass transfer adds: the 4 doubles of each state's record
+// that its 64 bytes do not hold (XferArgs::ext).
+constexpr size_t kExtBlockBytes = (size_t)kBlockStates * 4 * sizeof(double);
+
 // Workspace bytes the streamed shape needs for nrays rays: counters, chunk counts, ray records
 // and the arena at the per-ray budget (per_ray: kPerRayBytes, or kSurPerRayBytes for the
 // surrogate form).
@@ -1009,7 +1013,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
 
     // workspace carving; the surrogate form adds, per saved state, the network's inputs and
     // outputs (16 + 32 bytes)
-    const size_t per_ray = kPerRayBytes + (sur ? (size_t)kBudgetBlocksPerRay * kBlockStates * 48 : 0);
+    size_t per_ray = kPerRayBytes + (sur ? (size_t)kBudgetBlocksPerRay * kBlockStates * 48 : 0);
 
     // launch shape: the configured one, or automatic. RT_MIXED and RT_UNPOL overlap images of
     // 2^19 rays or more: streamed (chunks of about 2^15 rays, the geodesic at its own occupancy)
@@ -1030,6 +1034,12 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     // that hold a chunk each, with their own counters
     int rv = RT_OK, P = ovl ? plan_pieces(c, nrays, sur ? kSurPerRayBytes : kPerRayBytes) : 0, Kp = 0;
     const bool streamed = P > 0;
+    // the FP64 form in one pass: room for the transfer's records, unless a caller's workspace
+    // cannot hold one ray with them
+    bool ext = form == RT_FP64 && !ovl;
+    if (ext && c->ws && !c->ws_owned)
+        ext = c->ws_bytes > align_up(sizeof(Counters)) + 4 * kAlign + per_ray + kBudgetBlocksPerRay * kExtBlockBytes;
+    if (ext) per_ray += kBudgetBlocksPerRay * kExtBlockBytes;
     ChunkLayout L{nrays, 1, 1};
     if (streamed) {
         // contiguous ranges of each piece's longest-first order; the automatic shape takes finer
@@ -1060,7 +1070,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     // the layout {n, Kseq, 1} (chunk k from k (n / Kseq) + min(k, n % Kseq)), so that with the
     // longest-first order every chunk holds the same mix of lengths and none outgrows the
     // arena's per-ray budget
-    const size_t per_block = kBlockBytes + (sur ? (size_t)kBlockStates * 48 : 0);
+    const size_t per_block = kBlockBytes + (sur ? (size_t)kBlockStates * 48 : 0) + (ext ? kExtBlockBytes : 0);
     char *base = (char *)c->ws;
     Counters *ctr = (Counters *)base;
     size_t off = align_up(sizeof(Counters));
@@ -1083,6 +1093,11 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
         feat = (float4 *)(base + off);
         off = align_up(off + (size_t)nblocks * kBlockStates * sizeof(float4));
         sur_y = (float *)(base + off);
+    }
+    double *d_ext = nullptr;
+    if (ext) {
+        off = align_up(off + (size_t)nblocks * kBlockBytes);
+        d_ext = (double *)(base + off);
     }
 
     // ray order: longest first once a render of this camera has recorded its step counts, or,
@@ -1169,6 +1184,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
             XferArgs xa{cam, mod, ar, rec, ctr, n, o, d_out, d_status, d_depth};
             xa.pix_list = ray_list;
             xa.kt = KappaTables{c->d_syn, c->d_gl, c->d_gl + 8};
+            xa.ext = d_ext;
             if (sur) set_surrogate_args(c, xa, feat, sur_y);
             if (k == 0) CK(cudaEventRecord(c->ev[0], c->stream));
             launch_geodesic(ga, geo_grid, c->stream);

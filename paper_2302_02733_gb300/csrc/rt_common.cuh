@@ -107,10 +107,11 @@ struct KappaTables {
 };
 
 struct Counters {
-    // the first four are reset before every chunk of rays
+    // the first four are reset before every chunk of rays, and chain_next before every transfer
     unsigned long long geo_next, xfer_next;   // work-queue heads
     unsigned long long feat_next;             // queue of the surrogate's features pass
     unsigned long long arena_next;            // next free arena block
+    unsigned long long chain_next;            // queue of the transfer's Stokes chain
     unsigned long long feat_count;            // emitting points written by rt_render_features
     unsigned long long steps, points, emitting;
     unsigned int n_status[8];

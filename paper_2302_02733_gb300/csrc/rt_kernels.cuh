@@ -99,6 +99,8 @@ struct XferArgs {
     const int *pix_list;  // optional: the pixel of each global ray id (adaptive rendering)
     const JobDev *jobs;   // optional: a table of images (see GeoArgs)
     int njobs;
+    double *ext;          // FP64: 4 doubles per saved state for the points' records, or NULL (then one
+                          // kernel does the whole transfer)
 };
 
 // ---- batched rendering: many images in one persistent launch ----------------------------

@@ -373,16 +373,13 @@ __device__ __forceinline__ void taylor_inc(R tau, R aQ, R aV, R rQ, R rV, const 
     }
 }
 
-// One exact constant-coefficient step of dS/ds = J js - M S over ds on the compensated value
-// S + Slo (js scales the emissivities: 1/w^3 for the invariant form). Thin steps (the common
+// One exact constant-coefficient step of dS/ds = J - M S on the compensated value S + Slo, with M
+// and J times ds given. Thin steps (the common
 // case) form the increment by the Taylor series and add it without rounding loss; thick steps
 // fold Slo in and apply the closed form.
 template <typename R>
-__device__ void substep(const R cf[8], R ds, R js, R S[4], R Slo[4]) {
+__device__ void substep(R tau, R aQ, R aV, R rQ, R rV, const R J[4], R S[4], R Slo[4]) {
     typedef Mth<R> F;
-    R tau = cf[3] * ds, aQ = cf[4] * ds, aV = cf[5] * ds, rQ = cf[6] * ds, rV = cf[7] * ds;
-    R jds = js * ds;
-    R J[4] = {cf[0] * jds, cf[1] * jds, R(0), cf[2] * jds};
     R nrm = tau + fabs(aQ) + fabs(aV) + fabs(rQ) + fabs(rV);
     if (!(nrm > R(0.5))) {
         R acc[4];

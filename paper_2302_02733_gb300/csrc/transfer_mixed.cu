@@ -5,17 +5,24 @@
 #include "transfer_kernel.cuh"
 
 namespace prt {
+template <int CM, bool JOBS>
+static void launch_two(const XferArgs &a, int grid, cudaStream_t s) {
+    cudaMemsetAsync(&a.ctr->chain_next, 0, sizeof(unsigned long long), s);
+    constexpr int T = PointsCfg<float>::threads;
+    // grid counts blocks of kXferThreads
+    points_kernel<float, CM, JOBS><<<ray_grid((grid * kXferThreads + T - 1) / T, a.nrays, T / 32), T, 0, s>>>(a);
+    chain_kernel<float, float, JOBS><<<ray_grid(2 * grid, a.nrays, kXferThreads), kXferThreads, 0, s>>>(a);
+}
 void launch_transfer_mixed(const XferArgs &a, int coef, int grid, cudaStream_t s) {
-    grid = ray_grid(grid, a.nrays, kXferThreads);
     switch (coef) {
         case 0:
             if (a.jobs)
-                transfer_kernel<float, float, 0, true><<<grid, kXferThreads, 0, s>>>(a);
+                launch_two<0, true>(a, grid, s);
             else
-                transfer_kernel<float, float, 0><<<grid, kXferThreads, 0, s>>>(a);
+                launch_two<0, false>(a, grid, s);
             break;
-        case 1: transfer_kernel<float, float, 1><<<grid, kXferThreads, 0, s>>>(a); break;
-        case 2: transfer_kernel<float, float, 2><<<grid, kXferThreads, 0, s>>>(a); break;
+        case 1: launch_two<1, false>(a, grid, s); break;
+        case 2: launch_two<2, false>(a, grid, s); break;
         default: break;
     }
 }
@@ -48,16 +55,16 @@ static int func_regs(const void *f) {
     return a.numRegs;
 }
 int transfer_regs_mixed() {
-    int r = func_regs((const void *)transfer_kernel<float, float, 0>);
-    r = std::max(r, func_regs((const void *)transfer_kernel<float, float, 0, true>));
+    int r = func_regs((const void *)points_kernel<float, 0>);
+    r = std::max(r, func_regs((const void *)points_kernel<float, 0, true>));
     r = std::max(r, func_regs((const void *)transfer_kernel_staged<0>));
     r = std::max(r, func_regs((const void *)unpol_kernel<float>));
     return std::max(r, func_regs((const void *)unpol_kernel<float, true>));
 }
 int transfer_blocks_per_sm_mixed() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, transfer_kernel<float, float>, kXferThreads, 0) != cudaSuccess)
-        n = 1;
-    return n > 0 ? n : 1;
+    constexpr int T = PointsCfg<float>::threads;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, points_kernel<float>, T, 0) != cudaSuccess) n = 1;
+    return n > 0 ? n * (T / kXferThreads) : 1;
 }
 }  // namespace prt
