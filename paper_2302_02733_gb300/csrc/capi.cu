@@ -131,7 +131,7 @@ int rt_create(rt_ctx **out, int device, void *stream) {
     c->regs_per_sm = prop.regsPerMultiprocessor;
     bool ok = cudaMalloc(&c->d_stats, (8 + 4 * kStatBlocks) * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->d_sctab, kGeoTabBytes) == cudaSuccess &&
-              cudaMalloc(&c->d_syn, kSynTabBytes) == cudaSuccess && cudaMalloc(&c->d_gl, 16 * sizeof(double)) == cudaSuccess &&
+              cudaMalloc(&c->d_kap, kKapTabBytes) == cudaSuccess &&
               cudaMallocHost(&c->h_ctr, sizeof(Counters)) == cudaSuccess &&
               cudaStreamCreateWithFlags(&c->bstream, cudaStreamNonBlocking) == cudaSuccess;
     for (int i = 0; i < 3 && ok; i++) ok = cudaEventCreate(&c->ev[i]) == cudaSuccess;
@@ -142,7 +142,7 @@ int rt_create(rt_ctx **out, int device, void *stream) {
         return RT_ERR_CUDA;
     }
     memset(c->h_ctr, 0, sizeof(Counters));
-    if (launch_geo_tables(c->d_sctab, c->stream) != 0 || launch_kappa_tables(c->d_syn, c->d_gl, c->stream) != 0 || cudaStreamSynchronize(c->stream) != cudaSuccess) {
+    if (launch_geo_tables(c->d_sctab, c->stream) != 0 || launch_kappa_tables(c->d_kap, c->stream) != 0 || cudaStreamSynchronize(c->stream) != cudaSuccess) {
         cudaGetLastError();
         rt_destroy(c);
         return RT_ERR_CUDA;
@@ -177,8 +177,7 @@ int rt_destroy(rt_ctx *c) {
     cudaFree(c->d_stage_depth);
     cudaFree(c->d_stats);
     cudaFree(c->d_sctab);
-    cudaFree(c->d_syn);
-    cudaFree(c->d_gl);
+    cudaFree(c->d_kap);
     cudaFree(c->d_theta);
     cudaFree(c->d_wpk);
     cudaFree(c->d_tpk);
@@ -616,7 +615,7 @@ static int render_overlap(rt_ctx *c, int form, int coef, const Camera &cam, cons
         ga.njobs = njobs;
         XferArgs xa{cam, mod, ar[h], rec[h], ctr[h], n, o, d_out, d_status, d_depth};
         xa.pix_list = list;
-        xa.kt = KappaTables{c->d_syn, c->d_gl, c->d_gl + 8};
+        xa.kt = kappa_tables(c->d_kap);
         xa.jobs = jobs;
         xa.njobs = njobs;
         if (sur) set_surrogate_args(c, xa, feat[h], sur_y[h]);
@@ -834,7 +833,7 @@ static int render_streamed(rt_ctx *c, int form, int coef, const Camera &cam, con
                 const long long o = L.offset(a), n = L.offset(b - 1) + L.size(b - 1) - o;
                 XferArgs xa{cam, mod, ar, rec + o, ctr, n, o_p + o, d_out, d_status, d_depth};
                 xa.pix_list = list;
-                xa.kt = KappaTables{c->d_syn, c->d_gl, c->d_gl + 8};
+                xa.kt = kappa_tables(c->d_kap);
                 xa.jobs = jobs;
                 xa.njobs = njobs;
                 const int grid = q == cudaSuccess ? xf_grid_alone : xf_grid;
@@ -1183,7 +1182,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
             ga.steps_out = steps_out;
             XferArgs xa{cam, mod, ar, rec, ctr, n, o, d_out, d_status, d_depth};
             xa.pix_list = ray_list;
-            xa.kt = KappaTables{c->d_syn, c->d_gl, c->d_gl + 8};
+            xa.kt = kappa_tables(c->d_kap);
             xa.ext = d_ext;
             if (sur) set_surrogate_args(c, xa, feat, sur_y);
             if (k == 0) CK(cudaEventRecord(c->ev[0], c->stream));
@@ -1344,7 +1343,7 @@ int rt_kappa_coeffs(rt_ctx *c, const double *in, long long n, double *out) {
         if (!out_dev) d_out = (double *)tmp + 6 * n;
     }
     if (e == cudaSuccess) {
-        KappaTables T{c->d_syn, c->d_gl, c->d_gl + 8};
+        KappaTables T = kappa_tables(c->d_kap);
         launch_kappa_quad(T, d_in, d_out, n, c->nsm * 8, c->stream);
         e = cudaGetLastError();
     }

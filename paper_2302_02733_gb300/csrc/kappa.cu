@@ -1,35 +1,44 @@
 // Kappa-distribution coefficients by quadrature: the synchrotron-kernel tables and the batch
 // kernel behind rt_kappa_coeffs (one thread per point).
-#include <cmath>
-#include <vector>
-
 #include "kappa.cuh"
 #include "rt_kernels.cuh"
 
 namespace prt {
 
-// ln F, ln G, ln H at node i: trapezoid rule (step 1/100) on
-// F/x = int_0^inf e^{-x cosh t} cosh(5t/3)/cosh t dt, G/x = int e^{-x cosh t} cosh(2t/3) dt,
-// H = x int e^{-x cosh t} cosh(t/3) dt + int e^{-x cosh t} cosh(t/3)/cosh t dt.
-__global__ void synch_table_kernel(double *lnk) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kSynTab) return;
-    double x = exp(kSynLo + i * (kSynHi - kSynLo) / (kSynTab - 1));
-    const double h = 0.01;
-    double a = 0.0, b = 0.0, c = 0.0, d = 0.0;
-    for (int k = 0; k < 1000000; k++) {
-        double t = k * h, ch = cosh(t);
-        if (x * ch > 745.0) break;
-        double e = exp(-x * ch) * (k == 0 ? 0.5 : 1.0);
-        double c13 = cosh(t / 3.0);
-        a += e * cosh(5.0 * t / 3.0) / ch;
-        b += e * cosh(2.0 * t / 3.0);
-        c += e * c13;
-        d += e * c13 / ch;
+// Polynomials of K(x) e^x x^(-1/3) in t = -1 .. 1 on each interval of ln x: the values at the 8
+// Chebyshev nodes (one thread each, 16 intervals a block), their Chebyshev coefficients, and from
+// those the powers of t (the series falls off fast enough for the powers to lose nothing).
+constexpr int kSynPerBlock = 16;
+__global__ void __launch_bounds__(8 * kSynPerBlock) synch_poly_kernel(double *kern) {
+    __shared__ double f[3][kSynPerBlock][8], ch[3][kSynPerBlock][8];
+    const int li = threadIdx.x >> 3, j = threadIdx.x & 7, i = blockIdx.x * kSynPerBlock + li;
+    const double t = cospi((j + 0.5) * 0.125), lx = kSynLo + (i + 0.5 + 0.5 * t) * 0.125, x = exp(lx);
+    double k[3];
+    synch_kernels_scaled(x, k);
+    for (int m = 0; m < 3; m++) f[m][li][j] = k[m] * exp(-lx * (1.0 / 3.0));
+    __syncthreads();
+    for (int m = 0; m < 3; m++) {
+        double s = 0.0;
+        for (int n = 0; n < 8; n++) s += f[m][li][n] * cospi(j * (n + 0.5) * 0.125);
+        ch[m][li][j] = s * (j == 0 ? 0.125 : 0.25);
     }
-    lnk[i] = log(x * h * a);
-    lnk[kSynTab + i] = log(x * h * b);
-    lnk[2 * kSynTab + i] = log(x * h * c + h * d);
+    __syncthreads();
+    if (i >= kSynN || j >= 3) return;
+    double p[8] = {0}, a[8] = {1, 0, 0, 0, 0, 0, 0, 0}, b[8] = {0, 1, 0, 0, 0, 0, 0, 0};  // T_n, T_n+1
+    for (int n = 0; n < 8; n++) {
+        double c[8];
+        for (int q = 0; q < 8; q++) {
+            p[q] += ch[j][li][n] * a[q];
+            c[q] = (q > 0 ? 2.0 * b[q - 1] : 0.0) - a[q];
+        }
+        for (int q = 0; q < 8; q++) a[q] = b[q], b[q] = c[q];
+    }
+    for (int q = 0; q < 8; q++) kern[(3 * i + j) * 8 + q] = p[q];
+}
+
+__global__ void kap_node_kernel(KapNode *node) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < kKapN) node[k] = kap_node(kKapLo + k * kKapH);
 }
 
 __global__ void kappa_quad_kernel(KappaTables T, const double *in, double *out, long long n) {
@@ -42,29 +51,15 @@ __global__ void kappa_quad_kernel(KappaTables T, const double *in, double *out, 
     }
 }
 
-int launch_kappa_tables(double *lnk, double *gl, cudaStream_t s) {
-    // 8-point Gauss-Legendre rule on [-1, 1] (Newton iteration on P_8 from Chebyshev guesses)
-    const int n = 8;
-    double hb[16];
-    for (int i = 0; i < n; i++) {
-        double z = std::cos(kPi * (i + 0.75) / (n + 0.5)), dp = 1.0;
-        for (int it = 0; it < 100; it++) {
-            double p0 = 1.0, p1 = 0.0;
-            for (int j = 1; j <= n; j++) {
-                double p2 = p1;
-                p1 = p0;
-                p0 = ((2.0 * j - 1.0) * z * p1 - (j - 1.0) * p2) / j;
-            }
-            dp = n * (z * p0 - p1) / (z * z - 1.0);
-            double dz = p0 / dp;
-            z -= dz;
-            if (std::fabs(dz) < 1e-16) break;
-        }
-        hb[i] = z;
-        hb[8 + i] = 2.0 / ((1.0 - z * z) * dp * dp);
-    }
-    if (cudaMemcpyAsync(gl, hb, sizeof(hb), cudaMemcpyHostToDevice, s) != cudaSuccess) return -1;
-    synch_table_kernel<<<(kSynTab + 127) / 128, 128, 0, s>>>(lnk);
+KappaTables kappa_tables(const double *buf) {
+    return KappaTables{buf, reinterpret_cast<const KapNode *>(buf + 24 * kSynN)};
+}
+
+static_assert(kKapTabBytes == sizeof(double) * 24 * kSynN + sizeof(KapNode) * kKapN, "kappa tables' size");
+
+int launch_kappa_tables(double *buf, cudaStream_t s) {
+    synch_poly_kernel<<<(kSynN + kSynPerBlock - 1) / kSynPerBlock, 8 * kSynPerBlock, 0, s>>>(buf);
+    kap_node_kernel<<<(kKapN + 127) / 128, 128, 0, s>>>(reinterpret_cast<KapNode *>(buf + 24 * kSynN));
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

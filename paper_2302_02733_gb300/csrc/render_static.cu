@@ -90,7 +90,7 @@ int rt_render_static(rt_ctx *c, int form, void *out_iquv, uint8_t *status) {
     const int xf_b = c->rcfg.xfer_blocks_per_sm > 0 ? std::min(c->rcfg.xfer_blocks_per_sm, xf_max) : xf_max;
     launch_geodesic(ga, c->nsm * geo_b, c->stream);
     cudaEventRecord(c->ev[1], c->stream);
-    xa.kt = KappaTables{c->d_syn, c->d_gl, c->d_gl + 8};
+    xa.kt = kappa_tables(c->d_kap);
     const int coef = mod.edf == RT_EDF_KAPPA ? 1 : 0;
     if (form == RT_FP64)
         launch_transfer_fp64(xa, coef, c->nsm * xf_b, c->stream);

@@ -99,11 +99,11 @@ struct Model {
     double kappa;  // its index (> 3)
 };
 
-// Tables of the kappa quadrature (kappa.cuh): ln F, ln G, ln H and the Gauss-Legendre rule.
+// Tables of the kappa quadrature (kappa.cuh): the kernels' polynomials and the nodes.
+struct KapNode;
 struct KappaTables {
-    const double *lnk;  // [3][4096]
-    const double *glx;  // 8 nodes on [-1, 1]
-    const double *glw;  // and weights
+    const double *kern;   // [274][3][8]
+    const KapNode *node;  // [2000]
 };
 
 struct Counters {

@@ -37,8 +37,7 @@ struct rt_ctx {
     size_t stage_depth_bytes = 0;
     double *d_stats = nullptr;
     double *d_sctab = nullptr;  // the geodesic's sin and cos tables
-    double *d_syn = nullptr;    // ln F, ln G, ln H tables of the kappa quadrature
-    double *d_gl = nullptr;     // its Gauss-Legendre nodes and weights
+    double *d_kap = nullptr;    // tables of the kappa quadrature
     // surrogate MLP: parameters | Adam m | Adam v | gradient (FP32), tensor-core images, scalars
     float *d_theta = nullptr;
     void *d_wpk = nullptr, *d_tpk = nullptr, *d_mlpaux = nullptr;

@@ -177,8 +177,9 @@ int pipe_blocks_per_sm_fp64();
 int pipe_blocks_per_sm_mixed();
 
 // ---- kappa-distribution coefficients by quadrature (kappa.cuh) ---------------------------
-constexpr size_t kSynTabBytes = 3 * 4096 * sizeof(double);
-int launch_kappa_tables(double *lnk, double *gl16, cudaStream_t s);  // gl16: 8 nodes + 8 weights
+constexpr size_t kKapTabBytes = (24 * 274 + 8 * 2000) * sizeof(double);
+int launch_kappa_tables(double *buf, cudaStream_t s);  // kKapTabBytes
+KappaTables kappa_tables(const double *buf);
 void launch_kappa_quad(const KappaTables &T, const double *in, double *out, long long n, int grid, cudaStream_t s);
 
 // The blocks of a persistent launch over n rays: no more than take a ray each at its start. (With

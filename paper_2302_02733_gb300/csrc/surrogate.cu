@@ -407,7 +407,7 @@ int rt_surrogate_dataset(rt_ctx *c, const float box[8], long long n, uint64_t se
         b.lo[j] = box[j];
         b.hi[j] = box[4 + j];
     }
-    KappaTables T{c->d_syn, c->d_gl, c->d_gl + 8};
+    KappaTables T = kappa_tables(c->d_kap);
     sur_dataset_kernel<<<c->nsm * 8, 128, 0, c->stream>>>(T, b, seed, n, x, y, valid);
     SK(cudaGetLastError());
     SK(cudaStreamSynchronize(c->stream));
@@ -510,7 +510,7 @@ int rt_surrogate_coeffs(rt_ctx *c, const double *in, long long n, double *out, u
     float *yh = xn + 4 * n;
     unsigned char *ins = reinterpret_cast<unsigned char *>(yh + 8 * n);
     SurBox b = box_of(c->mlp_norm);
-    KappaTables T{c->d_syn, c->d_gl, c->d_gl + 8};
+    KappaTables T = kappa_tables(c->d_kap);
     int rv = RT_OK;
     sur_features_kernel<<<c->nsm * 8, 128, 0, c->stream>>>(in, n, b, xn, ins);
     if (cudaMemsetAsync(aux_err(c), 0, sizeof(unsigned), c->stream) != cudaSuccess) rv = RT_ERR_CUDA;
