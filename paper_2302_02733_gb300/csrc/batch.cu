@@ -148,7 +148,7 @@ int enqueue(rt_ctx *c, int form, const rt_batch_config &cfg, int njobs, long lon
     BK(cudaMemsetAsync(c->d_ready, 0xff, sizeof(int) * (size_t)nrays, s));
     launch_pool_init(c->pool, c->d_pctr, s);
     PipeArgs a{c->d_jobs, njobs, c->d_sctab, c->pool, c->d_brec, c->d_ready, c->d_pctr, nrays, cfg.geo_warps,
-               cfg.step_tile, cfg.geo_warps_odd > 0 ? cfg.geo_warps_odd : cfg.geo_warps};
+               cfg.step_tile, cfg.geo_warps_odd > 0 ? cfg.geo_warps_odd : cfg.geo_warps, c->d_therm};
     int grid = c->nsm * cfg.blocks_per_sm;
     if (form == RT_FP64)
         launch_pipe_fp64(a, grid, s);

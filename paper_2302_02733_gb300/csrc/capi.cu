@@ -132,6 +132,7 @@ int rt_create(rt_ctx **out, int device, void *stream) {
     bool ok = cudaMalloc(&c->d_stats, (8 + 4 * kStatBlocks) * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->d_sctab, kGeoTabBytes) == cudaSuccess &&
               cudaMalloc(&c->d_kap, kKapTabBytes) == cudaSuccess &&
+              cudaMalloc(&c->d_therm, kThermTabBytes) == cudaSuccess &&
               cudaMallocHost(&c->h_ctr, sizeof(Counters)) == cudaSuccess &&
               cudaStreamCreateWithFlags(&c->bstream, cudaStreamNonBlocking) == cudaSuccess;
     for (int i = 0; i < 3 && ok; i++) ok = cudaEventCreate(&c->ev[i]) == cudaSuccess;
@@ -142,7 +143,8 @@ int rt_create(rt_ctx **out, int device, void *stream) {
         return RT_ERR_CUDA;
     }
     memset(c->h_ctr, 0, sizeof(Counters));
-    if (launch_geo_tables(c->d_sctab, c->stream) != 0 || launch_kappa_tables(c->d_kap, c->stream) != 0 || cudaStreamSynchronize(c->stream) != cudaSuccess) {
+    if (launch_geo_tables(c->d_sctab, c->stream) != 0 || launch_kappa_tables(c->d_kap, c->stream) != 0 ||
+        launch_thermal_tables(c->d_therm, c->stream) != 0 || cudaStreamSynchronize(c->stream) != cudaSuccess) {
         cudaGetLastError();
         rt_destroy(c);
         return RT_ERR_CUDA;
@@ -178,6 +180,7 @@ int rt_destroy(rt_ctx *c) {
     cudaFree(c->d_stats);
     cudaFree(c->d_sctab);
     cudaFree(c->d_kap);
+    cudaFree(c->d_therm);
     cudaFree(c->d_theta);
     cudaFree(c->d_wpk);
     cudaFree(c->d_tpk);
@@ -616,6 +619,7 @@ static int render_overlap(rt_ctx *c, int form, int coef, const Camera &cam, cons
         XferArgs xa{cam, mod, ar[h], rec[h], ctr[h], n, o, d_out, d_status, d_depth};
         xa.pix_list = list;
         xa.kt = kappa_tables(c->d_kap);
+        xa.therm = c->d_therm;
         xa.jobs = jobs;
         xa.njobs = njobs;
         if (sur) set_surrogate_args(c, xa, feat[h], sur_y[h]);
@@ -834,6 +838,7 @@ static int render_streamed(rt_ctx *c, int form, int coef, const Camera &cam, con
                 XferArgs xa{cam, mod, ar, rec + o, ctr, n, o_p + o, d_out, d_status, d_depth};
                 xa.pix_list = list;
                 xa.kt = kappa_tables(c->d_kap);
+                xa.therm = c->d_therm;
                 xa.jobs = jobs;
                 xa.njobs = njobs;
                 const int grid = q == cudaSuccess ? xf_grid_alone : xf_grid;
@@ -1183,6 +1188,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
             XferArgs xa{cam, mod, ar, rec, ctr, n, o, d_out, d_status, d_depth};
             xa.pix_list = ray_list;
             xa.kt = kappa_tables(c->d_kap);
+            xa.therm = c->d_therm;
             xa.ext = d_ext;
             if (sur) set_surrogate_args(c, xa, feat, sur_y);
             if (k == 0) CK(cudaEventRecord(c->ev[0], c->stream));

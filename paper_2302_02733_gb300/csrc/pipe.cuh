@@ -303,9 +303,9 @@ __device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *sgw) {
 
 template <typename R, typename OutT>
 __global__ void __launch_bounds__(kPipeThreads, sizeof(R) == 4 ? 2 : 1) pipe_kernel(PipeArgs p) {
-    __shared__ R sgw[32];
+    __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
     __shared__ __align__(16) fx64 fxtab[2 * kFxTab];  // the geodesic's sin/cos table
-    fill_bessel_weights(sgw);
+    const R *sgw = thermal_weights(wsh, p.therm);
     load_fx_table(p.sctab, fxtab);
     __syncthreads();
     if ((int)(threadIdx.x >> 5) < ((blockIdx.x & 1) ? p.geo_warps_odd : p.geo_warps))

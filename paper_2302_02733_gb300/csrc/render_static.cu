@@ -91,6 +91,7 @@ int rt_render_static(rt_ctx *c, int form, void *out_iquv, uint8_t *status) {
     launch_geodesic(ga, c->nsm * geo_b, c->stream);
     cudaEventRecord(c->ev[1], c->stream);
     xa.kt = kappa_tables(c->d_kap);
+    xa.therm = c->d_therm;
     const int coef = mod.edf == RT_EDF_KAPPA ? 1 : 0;
     if (form == RT_FP64)
         launch_transfer_fp64(xa, coef, c->nsm * xf_b, c->stream);

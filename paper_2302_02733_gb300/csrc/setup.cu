@@ -29,6 +29,69 @@ void launch_x2_table(const GridModel &g, double *table, float *table_f, cudaStre
     x2_table_kernel<<<(n + 255) / 256, 256, 0, s>>>(g, table, table_f);
 }
 
+// The FP64 tables of ThermTab: on each segment the functions at the D + 1 Chebyshev nodes (one thread
+// each), their Chebyshev coefficients, and from those the powers of u.
+__device__ void bessel_ratio_values(double Te, double v[2]) {
+    // K_n(z) e^z = int_0^inf e^{-2 z sinh^2(t/2)} cosh(n t) dt by the trapezoid rule
+    const double z = 1.0 / Te, h = 0.125 * fmin(1.0, rsqrt(z));
+    double s0 = 0.5, s1 = 0.5, s2 = 0.5;
+    for (int k = 1; k < 100000; k++) {
+        const double t = k * h, sh = sinh(0.5 * t), e = 2.0 * z * sh * sh;
+        if (e > 2.0 * t + 60.0) break;
+        const double w = exp(-e), c = cosh(t);
+        s0 += w;
+        s1 += w * c;
+        s2 += w * (2.0 * c * c - 1.0);
+    }
+    v[0] = s0 / s2;
+    v[1] = s1 / s2;
+}
+__device__ void shcherbakov_values(double X, double v[2]) {
+    v[0] = shcherbakov_fX(X);
+    v[1] = 1.0 - 0.11 * log1p(0.035 * X);
+}
+
+constexpr int kThermPerBlock = 16;
+template <int D, void (*fn)(double, double *)>
+__global__ void therm_table_kernel(double *tab, int e0, int n) {
+    __shared__ double f[2][kThermPerBlock][D + 1], ch[2][kThermPerBlock][D + 1];
+    const int li = threadIdx.x / (D + 1), j = threadIdx.x % (D + 1), i = blockIdx.x * kThermPerBlock + li;
+    const double x = cospi((j + 0.5) / (D + 1));
+    double v[2];
+    fn(ldexp(1.0 + ((i & 15) + 0.5 + 0.5 * x) / 16.0, e0 + (i >> 4)), v);
+    f[0][li][j] = v[0];
+    f[1][li][j] = v[1];
+    __syncthreads();
+    for (int m = 0; m < 2; m++) {
+        double s = 0.0;
+        for (int q = 0; q <= D; q++) s += f[m][li][q] * cospi(j * (q + 0.5) / (D + 1));
+        ch[m][li][j] = s * (j == 0 ? 1.0 : 2.0) / (D + 1);
+    }
+    __syncthreads();
+    if (i >= n || j >= 2) return;
+    double p[D + 1], a[D + 1], b[D + 1];  // T_k and T_k+1 in powers of x = 2 u
+    for (int q = 0; q <= D; q++) p[q] = 0.0, a[q] = q == 0, b[q] = q == 1;
+    for (int k = 0; k <= D; k++) {
+        double c[D + 1];
+        for (int q = 0; q <= D; q++) {
+            p[q] += ch[j][li][k] * a[q];
+            c[q] = (q > 0 ? 2.0 * b[q - 1] : 0.0) - a[q];
+        }
+        for (int q = 0; q <= D; q++) a[q] = b[q], b[q] = c[q];
+    }
+    for (int q = 0; q <= D; q++) tab[(2 * i + j) * (D + 1) + q] = ldexp(p[q], q);
+}
+
+int launch_thermal_tables(double *buf, cudaStream_t s) {
+    typedef ThermTab T;
+    static_assert(T::nb % kThermPerBlock == 0 && T::ns % kThermPerBlock == 0, "whole blocks");
+    therm_table_kernel<T::db, bessel_ratio_values>
+        <<<T::nb / kThermPerBlock, kThermPerBlock * (T::db + 1), 0, s>>>(buf + T::bes, T::eb, T::nb);
+    therm_table_kernel<T::ds, shcherbakov_values>
+        <<<T::ns / kThermPerBlock, kThermPerBlock * (T::ds + 1), 0, s>>>(buf + T::shc, T::es, T::ns);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
 // Image statistics in two deterministic passes: each block takes a fixed contiguous range of
 // pixels, sums it with Kahan compensation per thread and a pairwise tree in shared memory, and
 // writes its partial sums; one block then adds the partials in block order. The epilogue forms

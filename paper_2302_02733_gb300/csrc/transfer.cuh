@@ -14,6 +14,7 @@
 #pragma once
 #include "camera.cuh"
 #include "ffloat.cuh"
+#include "polarmap.cuh"
 #include "rt_kernels.cuh"
 
 namespace prt {
@@ -43,8 +44,6 @@ struct Mth<double> {
     static __device__ __forceinline__ double floor_(double x) { return floor(x); }
     static __device__ __forceinline__ double fmod_(double x, double y) { return fmod(x, y); }
     static constexpr double jflush = 1e-250;  // emissivity below this carries no precision
-    static constexpr int taylor_max = 24;
-    static constexpr double taylor_tol = 1e-17;
     static constexpr double degen_D = 1e-9, degen_tp = 1e-3;
 };
 template <>
@@ -83,24 +82,37 @@ struct Mth<float> {
 //     c_0 = 1, c_1 = 1 + u^2/z, c_2 = 2 c_1^2 - 1, by the trapezoid rule on fixed nodes u_k = k h
 //     (the integrand is analytic in |Im u| < sqrt(2z), so the rule converges geometrically).
 //   K2 = K0 + (2/z) K1 for the series branch.
-template <typename R>
-struct BesselCfg;
-template <>
-struct BesselCfg<double> {
-    static constexpr int nser = 14, nq = 27;
-    static constexpr double h = 0.25;
-};
-template <>
-struct BesselCfg<float> {
+// In FP32 on every call; in FP64 only above the tables' end.
+struct BesselCfg {
     static constexpr int nser = 8, nq = 10;
     static constexpr float h = 0.5f;
 };
 
+// The series branch in FP64 (z < 2): above Theta = 2^20, where the tables end.
+__device__ __forceinline__ void bessel_k012_series(double z, double &k0, double &k1, double &k2) {
+    const double iz = 1.0 / z, hz = 0.5 * z, t = hz * hz, lg = log(hz) + 0.57721566490153286061;
+    double i0 = 0, s0 = 0, i1s = 0, s1 = 0, term0 = 1, term1 = 1, H = 0;
+    for (int k = 0; k < 14; k++) {
+        const double ik1 = 1.0 / (k + 1);
+        i0 += term0;
+        s0 += H * term0;
+        i1s += term1;
+        s1 += (2.0 * H + ik1) * term1;
+        H += ik1;
+        term0 *= t * ik1 * ik1;
+        term1 *= t * ik1 / (k + 2);
+    }
+    const double e = exp(z);
+    k0 = (s0 - lg * i0) * e;
+    k1 = (iz + lg * (hz * i1s) - 0.25 * z * s1) * e;
+    k2 = k0 + 2.0 * iz * k1;
+}
+
 // gw[k] = exp(-(k h)^2), halved at k = 0 (trapezoid end weight); kept in shared memory.
-template <typename R>
-__device__ __forceinline__ void bessel_k012_scaled(R z, const R *gw, R &k0, R &k1, R &k2) {
+__device__ __forceinline__ void bessel_k012_scaled(float z, const float *gw, float &k0, float &k1, float &k2) {
+    typedef float R;
     typedef Mth<R> F;
-    typedef BesselCfg<R> B;
+    typedef BesselCfg B;
     R iz = R(1) / z;
     if (z < R(2)) {
         R hz = R(0.5) * z, t = hz * hz;
@@ -164,6 +176,83 @@ __device__ __forceinline__ R shcherbakov_fX(R X) {
 }
 
 // ------------------------------------------------------------------------------------------
+// FP64 tables of functions of one positive variable: a polynomial on each sixteenth of an octave,
+// found from the exponent and the top four mantissa bits, in the rest of the mantissa (as
+// u = -1/2 .. 1/2, one FP64 instruction). Two functions to a segment, D + 1 coefficients each.
+//  - ThermTab::bes: K0/K2 and K1/K2 of z = 1/Theta for Theta from 2^-40 (1e-12) to 2^20;
+//  - ThermTab::shc: Shcherbakov's f(X) and 1 - 0.11 ln(1 + 0.035 X) for X from 2^-30 to 2^14.
+// 17 and 19 FP64 instructions in place of 27 reciprocal square roots (14 series terms at z < 2) and of
+// 11 transcendental functions; the FP64 pipe bounds the kernel. With fmks_y64 the FP64 instructions of
+// 32 states go from 1,721 to 1,343 and the points of a torus at 200^2 from 51 to 36 ms; an ADAF's
+// transfer at 64^2 from 16.4 to 9.5 ms. The functions have no singular point nearer than 16 segments,
+// so the fits converge as (1/66)^D; the values behind them are sums of positive terms.
+struct ThermTab {
+    static constexpr int db = 8, ds = 9;                    // degrees
+    static constexpr int eb = -40, nb = 60 * 16, es = -30, ns = 44 * 16;  // first octave, segments
+    static constexpr int bes = 0, shc = nb * 2 * (db + 1), size = shc + ns * 2 * (ds + 1);
+};
+static_assert(kThermTabBytes == ThermTab::size * sizeof(double), "thermal tables' size");
+
+// The segment of v >= 2^e0 and its variable u.
+__device__ __forceinline__ int therm_segment(double v, int e0, double &u) {
+    const long long b = __double_as_longlong(v);
+    u = __longlong_as_double((b << 4 & 0x000fffffffffffffll) | 0x3ff0000000000000ll) - 1.5;
+    return (int)(b >> 48) - ((1023 + e0) << 4);
+}
+template <int D>
+__device__ __forceinline__ void therm_eval(const double *t, double u, double &a, double &b) {
+    a = t[D];
+    b = t[2 * D + 1];
+#pragma unroll
+    for (int k = D - 1; k >= 0; k--) {
+        a = fma(a, u, t[k]);
+        b = fma(b, u, t[D + 1 + k]);
+    }
+}
+
+// Ratios K0/K2 and K1/K2 at 1/Theta. gw: in FP32 the quadrature's weights, in FP64 the tables.
+template <typename R>
+__device__ __forceinline__ void bessel_ratios(R Te, const R *gw, R &r0, R &r1) {
+    if constexpr (sizeof(R) == 8) {
+        double u;
+        const int i = therm_segment(Te, ThermTab::eb, u);
+        if (i < 0) {  // K_n(z)/K_2(z) -> 1 as z -> infinity
+            r0 = r1 = 1.0;
+            return;
+        }
+        if (i < ThermTab::nb) {
+            therm_eval<ThermTab::db>(gw + ThermTab::bes + i * 2 * (ThermTab::db + 1), u, r0, r1);
+            return;
+        }
+        double k0, k1, k2;
+        bessel_k012_series(1.0 / Te, k0, k1, k2);
+        r0 = k0 / k2;
+        r1 = k1 / k2;
+    } else {
+        R k0 = R(1), k1 = R(1), k2 = R(1);  // as z -> infinity
+        if (Te > R(1e-12)) bessel_k012_scaled(R(1) / Te, gw, k0, k1, k2);
+        r0 = k0 / k2;
+        r1 = k1 / k2;
+    }
+}
+
+// Shcherbakov's f(X) and g(X) = 1 - 0.11 ln(1 + 0.035 X).
+template <typename R>
+__device__ __forceinline__ void shcherbakov_fg(R X, const R *gw, R &f, R &g) {
+    typedef Mth<R> F;
+    if constexpr (sizeof(R) == 8) {
+        double u;
+        const int i = therm_segment(X, ThermTab::es, u);
+        if (i >= 0 && i < ThermTab::ns) {
+            therm_eval<ThermTab::ds>(gw + ThermTab::shc + i * 2 * (ThermTab::ds + 1), u, f, g);
+            return;
+        }
+    }
+    f = shcherbakov_fX(X);
+    g = R(1) - R(0.11) * F::log1p_(R(0.035) * X);
+}
+
+// ------------------------------------------------------------------------------------------
 // Thermal synchrotron coefficients in the fluid frame (cgs).
 // Emission: the Dexter (2016) fits with nu_c = (3/2) nu_B sin(th) Theta^2, x = nu/nu_c:
 //   j_I = n e^2 nu/(2 sqrt3 c Theta^2) 2.5651 (1 + 1.92 x^-1/3 + 0.9977 x^-2/3) e^{-1.8899 x^1/3},
@@ -194,16 +283,11 @@ __device__ __forceinline__ void thermal_coeffs(R ne, R Te, R B, R nu, R sth, R c
     R nuB = cB * B;
     R rb = nuB / nu;
     R X = Te * F::sqrt_(R(1.4142135623730951) * sth * R(1e3) * rb);
-    R k0, k1, k2;
-    if (Te > R(1e-12)) {
-        bessel_k012_scaled<R>(R(1) / Te, gw, k0, k1, k2);
-    } else {  // K_n(z)/K_2(z) -> 1 as z -> infinity
-        k0 = k1 = k2 = R(1);
-    }
-    R f = shcherbakov_fX(X);
-    R gX = R(1) - R(0.11) * F::log1p_(R(0.035) * X);
-    out[6] = cQ2 * ne * rb * rb / nu * sth * sth * f * (k1 / k2 + R(6) * Te);
-    out[7] = R(2) * cQ2 * ne * rb / nu * cth * (k0 / k2) * gX;
+    R r0, r1, f, gX;
+    bessel_ratios(Te, gw, r0, r1);
+    shcherbakov_fg(X, gw, f, gX);
+    out[6] = cQ2 * ne * rb * rb / nu * sth * sth * f * (r1 + R(6) * Te);
+    out[7] = R(2) * cQ2 * ne * rb / nu * cth * r0 * gX;
     if (sth < R(1e-12)) return;
     R nuc = R(1.5) * nuB * sth * Te * Te;
     R x = nu / nuc;
@@ -346,8 +430,18 @@ __device__ __forceinline__ void bmul(R aQ, R aV, R rQ, R rV, const R v[4], R o[4
     o[3] = aV * v[0] - rQ * v[2];
 }
 
+// 1/k, and the number of terms K of the FP64 series for ||M|| < 2^-b, b = 0 .. 31 (four bits each; at
+// b = 0 ||M|| is 1/2):
+// the least with 2^-bK / (K + 1)! <= 2^-57, so that what is left out is below an eighth of the last
+// place of the first term.
+__constant__ double kInv[16] = {0.,      1.,      1. / 2,  1. / 3,  1. / 4,  1. / 5,  1. / 6,  1. / 7,
+                                1. / 8,  1. / 9,  1. / 10, 1. / 11, 1. / 12, 1. / 13, 1. / 14, 1. / 15};
+constexpr unsigned long long kTerms0 = 0x444555667789bdffull, kTerms1 = 0x2222333333333344ull;
+
 // Increment of one constant-coefficient step by the Taylor series of the exponential applied
-// to the vector: acc = sum_k t_k, t_1 = J - M S, t_k = -M t_{k-1} / k.
+// to the vector: acc = sum_k t_k, t_1 = J - M S, t_k = -M t_{k-1} / k. In FP64 by Horner's rule with a
+// fixed number of terms, (1 - M/2 (1 - M/3 (..))) t_1: no division, comparison or sum beside the terms'
+// products (442 to 386 FP64 instructions for 32 states of the chain, 20.7 to 16.1 ms at 200^2).
 template <typename R>
 __device__ __forceinline__ void taylor_inc(R tau, R aQ, R aV, R rQ, R rV, const R J[4], const R S[4], R acc[4]) {
     typedef Mth<R> F;
@@ -358,18 +452,30 @@ __device__ __forceinline__ void taylor_inc(R tau, R aQ, R aV, R rQ, R rV, const 
         t[i] = J[i] - tau * S[i] - b[i];
         acc[i] = t[i];
     }
-    for (int k = 2; k <= F::taylor_max; k++) {
-        bmul(aQ, aV, rQ, rV, t, b);
-        R ik = R(1) / R(k);
-        R m = 0, sz = 0;
+    if constexpr (sizeof(R) == 8) {
+        const double nrm = tau + fabs(aQ) + fabs(aV) + fabs(rQ) + fabs(rV);
+        const int e = 1022 - (int)((unsigned)__double2hiint(nrm) >> 20 & 0x7ffu);  // nrm < 2^-e (nrm <= 1/2: e >= 0)
+        const int K = e > 31 ? (e > 57 ? 1 : 2) : (int)((e < 16 ? kTerms0 >> (4 * (e < 0 ? 0 : e)) : kTerms1 >> (4 * (e - 16))) & 15ull);
+        for (int k = K; k >= 2; k--) {
+            const double ik = kInv[k];
+            bmul(aQ, aV, rQ, rV, acc, b);
 #pragma unroll
-        for (int i = 0; i < 4; i++) {
-            t[i] = -(tau * t[i] + b[i]) * ik;
-            acc[i] += t[i];
-            m = fmax(m, fabs(t[i]));
-            sz = fmax(sz, fabs(acc[i]) + fabs(S[i]));
+            for (int i = 0; i < 4; i++) acc[i] = fma(-ik, fma(tau, acc[i], b[i]), t[i]);
         }
-        if (m <= F::taylor_tol * sz) break;
+    } else {
+        for (int k = 2; k <= F::taylor_max; k++) {
+            bmul(aQ, aV, rQ, rV, t, b);
+            R ik = R(1) / R(k);
+            R m = 0, sz = 0;
+    #pragma unroll
+            for (int i = 0; i < 4; i++) {
+                t[i] = -(tau * t[i] + b[i]) * ik;
+                acc[i] += t[i];
+                m = fmax(m, fabs(t[i]));
+                sz = fmax(sz, fabs(acc[i]) + fabs(S[i]));
+            }
+            if (m <= F::taylor_tol * sz) break;
+        }
     }
 }
 
@@ -573,49 +679,32 @@ __device__ __forceinline__ R fmks_theta_w(const GridModel &g, R w, R x2, R *dth2
     return R(0.5 * kPi) + fmks_mu(g, w, x2 - R(0.5), dth2, thj_m_thg);
 }
 
-// y = X2 - 1/2 of the point at polar angle th (mu = th - pi/2, formed before rounding to R):
+// y = X2 - 1/2 of the point at polar angle th (mu = th - pi/2, formed before rounding to FP32):
 // a table guess in (w, theta), then Newton on mu.
-template <typename R>
-__device__ __forceinline__ R fmks_y(const GridModel &g, R w, R th, R mu) {
-    R fw = w * R(kX2TabW - 1);
-    R ft = th * R((kX2TabT - 1) / kPi);
-    int iw, it;
-    R tw, tt;
-    if constexpr (sizeof(R) == 4) {  // fw in [0, 63], ft in [0, 1023]: no conversion instructions
-        iw = min(max(floor_small(fw), 0), kX2TabW - 2);
-        it = min(max(floor_small(ft), 0), kX2TabT - 2);
-        tw = fw - i2f_small(iw);
-        tt = ft - i2f_small(it);
-    } else {
-        iw = min(max((int)fw, 0), kX2TabW - 2);
-        it = min(max((int)ft, 0), kX2TabT - 2);
-        tw = fw - R(iw);
-        tt = ft - R(it);
-    }
-    R x00, x01, x10, x11;
-    if (sizeof(R) == 8) {
-        const double *T = g.x2_table;
-        x00 = R(T[iw * kX2TabT + it]), x01 = R(T[iw * kX2TabT + it + 1]);
-        x10 = R(T[(iw + 1) * kX2TabT + it]), x11 = R(T[(iw + 1) * kX2TabT + it + 1]);
-    } else {
-        const float *T = g.x2_table_f;
-        x00 = R(T[iw * kX2TabT + it]), x01 = R(T[iw * kX2TabT + it + 1]);
-        x10 = R(T[(iw + 1) * kX2TabT + it]), x11 = R(T[(iw + 1) * kX2TabT + it + 1]);
-    }
-    R y = (R(1) - tw) * ((R(1) - tt) * x00 + tt * x01) + tw * ((R(1) - tt) * x10 + tt * x11) - R(0.5);
+__device__ __forceinline__ float fmks_y(const GridModel &g, float w, float th, float mu) {
+    float fw = w * float(kX2TabW - 1);
+    float ft = th * float((kX2TabT - 1) / kPi);
+    // fw in [0, 63], ft in [0, 1023]: no conversion instructions
+    int iw = min(max(floor_small(fw), 0), kX2TabW - 2);
+    int it = min(max(floor_small(ft), 0), kX2TabT - 2);
+    float tw = fw - i2f_small(iw);
+    float tt = ft - i2f_small(it);
+    const float *T = g.x2_table_f;
+    float x00 = T[iw * kX2TabT + it], x01 = T[iw * kX2TabT + it + 1];
+    float x10 = T[(iw + 1) * kX2TabT + it], x11 = T[(iw + 1) * kX2TabT + it + 1];
+    float y = (1.0f - tw) * ((1.0f - tt) * x00 + tt * x01) + tw * ((1.0f - tt) * x10 + tt * x11) - 0.5f;
     // the bilinear table guess is within 1.3e-5 of the root in y (a cell is 1/n2 = 7.8e-3); one
-    // Newton step takes that below 1e-9 and a second to FP64's resolution. FP32 takes two as
-    // well: after one the result still depends on how the guess was rounded, which differs
-    // between the kernels this is inlined into (the single, batched and staged transfers give
-    // bit-identical mixed images only after the second)
+    // Newton step takes that below 1e-9. Two all the same: after one the result still depends on how
+    // the guess was rounded, which differs between the kernels this is inlined into (the single,
+    // batched and staged transfers give bit-identical mixed images only after the second)
     const int iters = 2;
 #pragma unroll
     for (int k = 0; k < iters; k++) {
-        R d;
-        R f = fmks_mu(g, w, y, &d, (R *)nullptr) - mu;
+        float d;
+        float f = fmks_mu(g, w, y, &d, (float *)nullptr) - mu;
         y -= f / d;
     }
-    return fmin(fmax(y, R(-0.5)), R(0.5));
+    return fmin(fmax(y, -0.5f), 0.5f);
 }
 
 // Corner index and fraction of one axis of the trilinear fetch, from an approximate cell
@@ -649,6 +738,7 @@ struct GridCell {
     int i0, j0, k0, k1;
     R r, w, y;      // r in R, the FMKS blend weight and y = X2 - 1/2
     R w1, w2, w3;   // trilinear fractions
+    R dth2, dd;     // FP64: d theta / d X2 and theta_j - theta_g
 };
 
 // false outside r_in <= r <= r_out
@@ -710,7 +800,7 @@ __device__ __forceinline__ bool grid_cell(const GridModel &g, double rd, double 
         w1 = F::log1p_(R(rd * g.x1_irc[i0] - 1.0)) / pick<R>(g.dx1, g.f_dx1);
         cell_axis(g.n1, i0, w1);
         // polar: y = X2 - 1/2; fj = y n2 + (n2 - 1)/2, fraction about the half-integer j0 - (n2 - 1)/2
-        y = fmks_y(g, w, th, R(thd - 0.5 * kPi));
+        y = fmks_y64(g, w, th, thd - 0.5 * kPi, c.dth2, c.dd);
         R t = y * R(g.n2), c2 = R(0.5 * (g.n2 - 1));
         j0 = (int)F::floor_(t + c2);
         j0 = min(max(j0, 0), g.n2 - 2);
@@ -777,8 +867,8 @@ __device__ __forceinline__ void grid_state(const GridModel &g, const KS<R> &m, c
     const R r = c.r;
     R rho = P[0], uu = P[1];
     if (!(rho > R(0)) || !(uu > R(0))) return;
-    R dth2, dd;
-    fmks_mu(g, c.w, c.y, &dth2, &dd);
+    R dth2 = c.dth2, dd = c.dd;
+    if (sizeof(R) == 4) fmks_mu(g, c.w, c.y, &dth2, &dd);
     R dth1 = -pick<R>(g.mks_smooth, g.f_mks_smooth) * c.w * dd;
     R Ut[4] = {R(0), r * P[2], dth1 * P[2] + dth2 * P[3], P[4]};
     R Bi[4] = {R(0), r * P[5], dth1 * P[5] + dth2 * P[6], P[7]};

@@ -550,22 +550,23 @@ __device__ __forceinline__ void xfer_zero(long long pix, void *out, void *depth)
     }
 }
 
-// Bessel-quadrature weights exp(-(k h)^2) (halved at k = 0) into shared memory.
-template <typename R>
-__device__ __forceinline__ void fill_bessel_weights(R *sgw) {
-    typedef Mth<R> F;
-    if (threadIdx.x < BesselCfg<R>::nq) {
-        R u = R(threadIdx.x) * BesselCfg<R>::h;
-        sgw[threadIdx.x] = F::exp_(-u * u) * (threadIdx.x == 0 ? R(0.5) : R(1));
+// What the thermal coefficients read: in FP32 the Bessel quadrature's weights exp(-(k h)^2) (halved at
+// k = 0), put into shared memory here, in FP64 the tables in global memory.
+__device__ __forceinline__ const float *thermal_weights(float *sgw, const double *) {
+    if (threadIdx.x < BesselCfg::nq) {
+        float u = float(threadIdx.x) * BesselCfg::h;
+        sgw[threadIdx.x] = expf(-u * u) * (threadIdx.x == 0 ? 0.5f : 1.0f);
     }
+    return sgw;
 }
+__device__ __forceinline__ const double *thermal_weights(double *, const double *tab) { return tab; }
 
 // JOBS: the rays run over a table of images (p.jobs), each with its own camera, model and
 // outputs; otherwise over the one image of p.cam, p.model, p.out.
 template <typename R, typename OutT, int CM = 0, bool JOBS = false>
 __global__ void __launch_bounds__(kXferThreads, sizeof(R) == 4 ? 4 : 1) transfer_kernel(XferArgs p) {
-    __shared__ R sgw[32];
-    fill_bessel_weights(sgw);
+    __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
+    const R *sgw = thermal_weights(wsh, p.therm);
     __syncthreads();
     long long ray = -1;
     int blk = -1, slot = 0, n = 0, rstat = 0, job = 0;
@@ -724,8 +725,8 @@ struct PointsCfg<double> {
 // handed down lane by lane.
 template <typename R, int CM = 0, bool JOBS = false>
 __global__ void __launch_bounds__(PointsCfg<R>::threads, PointsCfg<R>::blocks) points_kernel(XferArgs p) {
-    __shared__ R sgw[32];
-    fill_bessel_weights(sgw);
+    __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
+    const R *sgw = thermal_weights(wsh, p.therm);
     __syncthreads();
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -967,7 +968,7 @@ __global__ void __launch_bounds__(kXferThreads, 4) transfer_kernel_staged(XferAr
     __shared__ R sgw[32];
     __shared__ __align__(128) float4 stc[kXferThreads * 16];
     __shared__ __align__(8) unsigned long long bars[kXferThreads];
-    fill_bessel_weights(sgw);
+    thermal_weights(sgw, p.therm);
     const uint32_t bar = smem_u32(&bars[threadIdx.x]);
     float4 *slot_s = stc + threadIdx.x * 16;
     const uint32_t slot_a = smem_u32(slot_s);
