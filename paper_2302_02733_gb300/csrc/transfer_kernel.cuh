@@ -1167,116 +1167,107 @@ __global__ void __launch_bounds__(kXferThreads) sur_features_pass(XferArgs p) {
 // (the ray's fluid-frame direction is -K - w u, b is spatial in that frame), j_I and a_I, and the
 // exact step I <- I e^-tau + (j ds / w^3) (1 - e^-tau)/tau, added as the increment
 // (J - tau I) (1 - e^-tau)/tau with TwoSum compensation. Output: one value per pixel.
+// One warp per ray, one lane per state of an arena block (as points_kernel); the increments of the
+// block's emitting states then follow one another, every lane adding the value that the state's lane
+// holds (11 instructions a state). With one lane per ray the states of a ray were a serial chain of a
+// point's whole evaluation each, and 16,384 rays filled a ninth of the chip: a torus at 128^2 took
+// 7.1 ms, now 0.78, at 1024^2 34.8 (256 threads and 3 blocks, with or without a barrier per block of
+// states, 34.7 and 36.0; 128 threads and 4 blocks 39.8).
 template <typename R, bool JOBS = false>
-__global__ void __launch_bounds__(kXferThreads, 4) unpol_kernel(XferArgs p) {
+__global__ void __launch_bounds__(kXferThreads, 6) unpol_kernel(XferArgs p) {
     typedef Mth<R> F;
-    // the ray's camera constants: p.cam's, or (JOBS) its image's
-    R a = pick<R>(p.cam.a, p.cam.f_a), nu_obs = pick<R>(p.cam.nu_obs, p.cam.f_nu_obs),
-      L = pick<R>(p.cam.L_unit, p.cam.f_L_unit);
-    long long ray = -1;
-    int blk = -1, slot = 0, n = 0, rstat = 0, job = 0;
-    bool live = false, drained = false;
-    R I = 0, Ilo = 0;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
     unsigned long long my_pts = 0, my_emit = 0;
-    auto gid_of = [&](long long r) { return p.pix_list ? (long long)p.pix_list[r + p.ray_offset] : r + p.ray_offset; };
-    // this ray's pixel index and its image's outputs
-    auto target = [&](long long &pix, R *&out, uint8_t *&status) {
-        int ix, iy;
-        if (JOBS) {
-            const JobDev &J = p.jobs[job];
-            ray_pixel(gid_of(ray) - J.ray_begin, J.cam.nx, J.cam.ny, ix, iy);
-            pix = (long long)iy * J.cam.nx + ix;
-            out = reinterpret_cast<R *>(J.out);
-            status = J.status;
-        } else {
-            map_pixel(p.pix_list, ray + p.ray_offset, p.cam.nx, p.cam.ny, ix, iy);
-            pix = (long long)iy * p.cam.nx + ix;
-            out = reinterpret_cast<R *>(p.out);
-            status = p.status;
-        }
-    };
+    const JobDev *J = nullptr;
+    long long ray = 0, gid = 0;
+    int N = 0, base = -1, blk = -1, rstat = 0;  // as in points_kernel
+    bool drained = false;
+    R I = 0, Ilo = 0;
     for (;;) {
-        bool want = !live && !drained;
-        unsigned long long t = warp_pop(&p.ctr->xfer_next, want);
-        if (want) {
-            if (t < (unsigned long long)p.nrays) {
+        if (base < 0 && !drained) {
+            unsigned long long t = 0;
+            if (lane == 0) t = atomicAdd(&p.ctr->xfer_next, 1ull);
+            t = __shfl_sync(full, t, 0);
+            drained = t >= (unsigned long long)p.nrays;
+            if (!drained) {
                 ray = (long long)t;
-                if (JOBS) {
-                    job = find_job(p.jobs, p.njobs, gid_of(ray));
-                    const Camera &cj = p.jobs[job].cam;
-                    a = pick<R>(cj.a, cj.f_a);
-                    nu_obs = pick<R>(cj.nu_obs, cj.f_nu_obs);
-                    L = pick<R>(cj.L_unit, cj.f_L_unit);
-                }
-                RayRecord rec = p.rec[ray];
+                const RayRecord rec = p.rec[ray];
+                gid = p.pix_list ? (long long)p.pix_list[ray + p.ray_offset] : ray + p.ray_offset;
+                if (JOBS) J = p.jobs + find_job(p.jobs, p.njobs, gid);
                 rstat = rec.status;
-                if (rec.nstates >= 2) {
-                    blk = rec.last_block;
-                    slot = (rec.nstates - 1) % kBlockStates;
-                    n = rec.nstates - 1;
-                    I = Ilo = R(0);
-                    live = true;
-                } else {
-                    long long pix;
-                    R *out;
-                    uint8_t *status;
-                    target(pix, out, status);
-                    out[pix] = R(0);
-                    if (status) status[pix] = (uint8_t)rstat;
+                N = max(rec.nstates - 1, 0);
+                blk = rec.last_block;
+                base = N / kBlockStates * kBlockStates;
+                if (base == N && N > 0) {  // the last block holds the last state alone
+                    base -= kBlockStates;
+                    blk = p.arena.prev[blk];
                 }
-            } else {
-                drained = true;
+                I = Ilo = R(0);
             }
         }
-        if (__all_sync(0xffffffffu, !live && drained)) break;
-        if (!live) continue;
-        if (--slot < 0) {
-            blk = p.arena.prev[blk];
-            slot = kBlockStates - 1;
-        }
-        n--;
-        const double4_32a *src = reinterpret_cast<const double4_32a *>(p.arena.states + (long long)blk * kBlockStates + slot);
-        double4_32a q0 = src[0], q1 = src[1];
-        R r = to_real<R>(q0.x), th = to_real<R>(q0.y), ph = to_real<R>(q0.z);
-        R K[4] = {to_real<R>(q0.w), to_real<R>(q1.x), to_real<R>(q1.y), to_real<R>(q1.z)};
-        R h = fabs(to_real<R>(q1.w));
-        KS<R> m;
-        m.eval(a, r, th);
-        Plasma<R> pl;
-        const Model &mdl = JOBS ? p.jobs[job].model : p.model;
-        if (mdl.kind == 1)
-            adaf_plasma(mdl.adaf, a, m, r, pl);
-        else
-            grid_plasma(mdl.grid, m, q0.x, q0.y, q0.z, pl);
-        if (pl.valid) {
-            R w = m.dot(K, pl.u);
-            R kp[4], bn[4];
-            R bs = fmax(fmax(fabs(pl.b[0]), fabs(pl.b[1])), fmax(fabs(pl.b[2]), fabs(pl.b[3])));
-            R ibs = bs > R(0) ? R(1) / bs : R(0);
+        if (drained) break;
+        if (base < 0) continue;
+        const Camera &c = JOBS ? J->cam : p.cam;
+        const int prev = base > 0 ? p.arena.prev[blk] : -1;
+        bool valid = false;
+        R tau = 0, Jn = 0, ph1 = 0;
+        if (base + lane < N) {
+            const double4_32a *src = reinterpret_cast<const double4_32a *>(p.arena.states + (long long)blk * kBlockStates + lane);
+            const double4_32a q0 = src[0], q1 = src[1];
+            R r = to_real<R>(q0.x), th = to_real<R>(q0.y);
+            R K[4] = {to_real<R>(q0.w), to_real<R>(q1.x), to_real<R>(q1.y), to_real<R>(q1.z)};
+            R h = fabs(to_real<R>(q1.w));
+            KS<R> m;
+            m.eval(pick<R>(c.a, c.f_a), r, th);
+            Plasma<R> pl;
+            const Model &mdl = JOBS ? J->model : p.model;
+            if (mdl.kind == 1)
+                adaf_plasma(mdl.adaf, pick<R>(c.a, c.f_a), m, r, pl);
+            else
+                grid_plasma(mdl.grid, m, q0.x, q0.y, q0.z, pl);
+            valid = pl.valid;
+            if (valid) {
+                R w = m.dot(K, pl.u);
+                R kp[4], bn[4];
+                R bs = fmax(fmax(fabs(pl.b[0]), fabs(pl.b[1])), fmax(fabs(pl.b[2]), fabs(pl.b[3])));
+                R ibs = bs > R(0) ? R(1) / bs : R(0);
 #pragma unroll
-            for (int i = 0; i < 4; i++) {
-                kp[i] = -K[i] - w * pl.u[i];
-                bn[i] = pl.b[i] * ibs;
+                for (int i = 0; i < 4; i++) {
+                    kp[i] = -K[i] - w * pl.u[i];
+                    bn[i] = pl.b[i] * ibs;
+                }
+                R bb = m.dot(bn, bn), kk = m.dot(kp, kp), bk = m.dot(bn, kp);
+                R sth = (bb > R(0) && kk > R(0)) ? F::sqrt_(fmax(bb - bk * bk / kk, R(0)) / bb) : R(0);
+                R jI, aI;
+                thermal_jI_aI(pl.ne, pl.Te, pl.B, w * pick<R>(c.nu_obs, c.f_nu_obs), sth, jI, aI);
+                R ds = w * h * pick<R>(c.L_unit, c.f_L_unit);
+                tau = aI * ds;
+                Jn = jI * ds / (w * w * w);
+                ph1 = phi1(tau);
             }
-            R bb = m.dot(bn, bn), kk = m.dot(kp, kp), bk = m.dot(bn, kp);
-            R sth = (bb > R(0) && kk > R(0)) ? F::sqrt_(fmax(bb - bk * bk / kk, R(0)) / bb) : R(0);
-            R jI, aI;
-            thermal_jI_aI(pl.ne, pl.Te, pl.B, w * nu_obs, sth, jI, aI);
-            R ds = w * h * L, tau = aI * ds;
-            R J = jI * ds / (w * w * w);
-            two_sum_add(I, Ilo, (J - tau * I) * phi1(tau));
-            my_emit++;
+            my_pts++;
+            my_emit += valid;
         }
-        my_pts++;
-        if (n == 0) {
-            long long pix;
-            R *out;
-            uint8_t *status;
-            target(pix, out, status);
-            out[pix] = I + Ilo;
+        for (unsigned em = __ballot_sync(full, valid); em;) {
+            const int j = 31 - __clz(em);
+            em ^= 1u << j;
+            const R tj = __shfl_sync(full, tau, j), Jj = __shfl_sync(full, Jn, j), pj = __shfl_sync(full, ph1, j);
+            two_sum_add(I, Ilo, (Jj - tj * I) * pj);
+        }
+        if (base == 0 && lane == 0) {
+            int ix, iy;
+            if (JOBS)
+                ray_pixel(gid - J->ray_begin, c.nx, c.ny, ix, iy);
+            else
+                map_pixel(p.pix_list, ray + p.ray_offset, c.nx, c.ny, ix, iy);
+            const long long pix = (long long)iy * c.nx + ix;
+            reinterpret_cast<R *>(JOBS ? J->out : p.out)[pix] = N > 0 ? I + Ilo : R(0);
+            uint8_t *status = JOBS ? J->status : p.status;
             if (status) status[pix] = (uint8_t)rstat;
-            live = false;
         }
+        blk = prev;
+        base -= kBlockStates;
     }
     if (my_pts) atomicAdd(&p.ctr->points, my_pts);
     if (my_emit) atomicAdd(&p.ctr->emitting, my_emit);

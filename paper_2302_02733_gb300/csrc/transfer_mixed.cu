@@ -36,7 +36,7 @@ int transfer_blocks_per_sm_staged() {
     return n > 0 ? n : 1;
 }
 void launch_unpol(const XferArgs &a, int grid, cudaStream_t s) {
-    grid = ray_grid(grid, a.nrays, kXferThreads);
+    grid = ray_grid(grid, a.nrays, kXferThreads / 32);
     if (a.jobs)
         unpol_kernel<float, true><<<grid, kXferThreads, 0, s>>>(a);
     else
