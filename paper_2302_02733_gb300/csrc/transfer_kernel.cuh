@@ -1091,74 +1091,82 @@ __global__ void __launch_bounds__(kXferThreads, 4) transfer_kernel_staged(XferAr
     if (my_emit) atomicAdd(&p.ctr->emitting, my_emit);
 }
 
-// The surrogate form's features pass: walk each ray's saved states as the transfer will and
-// write, for every emitting state, the network's normalised inputs (f mapped from the box to
-// [-1, 1]); other states get zeros. Same arithmetic as the transfer's own feature evaluation.
+// The surrogate form's features pass: for every emitting saved state the network's normalised inputs
+// (f mapped from the box to [-1, 1]); other states get zeros. Same arithmetic as the transfer's own
+// feature evaluation. One warp per ray, one lane per state of an arena block (as points_kernel).
 template <typename R>
-__global__ void __launch_bounds__(kXferThreads) sur_features_pass(XferArgs p) {
+__global__ void __launch_bounds__(kXferThreads, 5) sur_features_pass(XferArgs p) {
     const Camera &c = p.cam;
     const R a = pick<R>(c.a, c.f_a), nu_obs = pick<R>(c.nu_obs, c.f_nu_obs);
-    long long ray = -1, row = 0;
-    int blk = -1, slot = 0, n = 0;
-    bool live = false, drained = false;
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    long long row = 0;
+    int N = 0, base = -1, blk = -1;  // as in points_kernel
     for (;;) {
-        bool want = !live && !drained;
-        unsigned long long t = warp_pop(&p.ctr->feat_next, want);
-        if (want) {
-            if (t < (unsigned long long)p.nrays) {
-                ray = (long long)t;
-                RayRecord rec = p.rec[ray];
-                if (rec.nstates >= 2) {
-                    blk = rec.last_block;
-                    slot = (rec.nstates - 1) % kBlockStates;
-                    n = rec.nstates - 1;
-                    live = true;
-                    // compact rows: the ray's n states take n consecutive rows
-                    if (p.sur_row) row = (long long)atomicAdd(&p.ctr->sur_rows, (unsigned long long)n);
-                }
-            } else {
-                drained = true;
+        if (base < 0) {
+            unsigned long long t = 0;
+            if (lane == 0) t = atomicAdd(&p.ctr->feat_next, 1ull);
+            t = __shfl_sync(full, t, 0);
+            if (t >= (unsigned long long)p.nrays) break;
+            const RayRecord rec = p.rec[t];
+            if (rec.nstates < 2) continue;
+            N = rec.nstates - 1;
+            blk = rec.last_block;
+            base = N / kBlockStates * kBlockStates;
+            if (base == N) {  // the last block holds the last state alone
+                base -= kBlockStates;
+                blk = p.arena.prev[blk];
+            }
+            // compact rows: the ray's N states take N consecutive rows
+            if (p.sur_row) {
+                if (lane == 0) row = (long long)atomicAdd(&p.ctr->sur_rows, (unsigned long long)N);
+                row = __shfl_sync(full, row, 0);
             }
         }
-        if (__all_sync(0xffffffffu, !live && drained)) break;
-        if (!live) continue;
-        if (--slot < 0) {
-            blk = p.arena.prev[blk];
-            slot = kBlockStates - 1;
-        }
-        n--;
-        const double4_32a *src = reinterpret_cast<const double4_32a *>(p.arena.states + (long long)blk * kBlockStates + slot);
-        double4_32a q0 = src[0], q1 = src[1];
-        R r = to_real<R>(q0.x), th = to_real<R>(q0.y), ph = to_real<R>(q0.z);
-        R K[4] = {to_real<R>(q0.w), to_real<R>(q1.x), to_real<R>(q1.y), to_real<R>(q1.z)};
-        KS<R> m;
-        m.eval(a, r, th);
-        Plasma<R> pl;
-        if (p.model.kind == 1)
-            adaf_plasma(p.model.adaf, a, m, r, pl);
-        else
-            grid_plasma(p.model.grid, m, q0.x, q0.y, q0.z, pl);
-        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (pl.valid) {
-            R e1[4], e2[4], w, sth, cth;
-            fluid_tetrad(m, K, pl.u, pl.b, e1, e2, w, sth, cth);
-            float f[4], xn[4];
-            sur_features_r<R>(pl.Te, pl.B, w * nu_obs, sth, cth, R(p.model.kappa), f);
-            if (p.feat_raw) {
-                unsigned long long k = atomicAdd(&p.ctr->feat_count, 1ull);
-                if ((long long)k < p.feat_cap) p.feat_raw[k] = make_float4(f[0], f[1], f[2], f[3]);
-            }
+        const int prev = base > 0 ? p.arena.prev[blk] : -1;
+        const bool act = base + lane < N;
+        const long long st = (long long)blk * kBlockStates + lane;
+        bool valid = false;
+        float f[4];
+        if (act) {
+            const double4_32a *src = reinterpret_cast<const double4_32a *>(p.arena.states + st);
+            const double4_32a q0 = src[0], q1 = src[1];
+            R r = to_real<R>(q0.x), th = to_real<R>(q0.y);
+            R K[4] = {to_real<R>(q0.w), to_real<R>(q1.x), to_real<R>(q1.y), to_real<R>(q1.z)};
+            KS<R> m;
+            m.eval(a, r, th);
+            Plasma<R> pl;
+            if (p.model.kind == 1)
+                adaf_plasma(p.model.adaf, a, m, r, pl);
+            else
+                grid_plasma(p.model.grid, m, q0.x, q0.y, q0.z, pl);
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            valid = pl.valid;
+            if (valid) {
+                R e1[4], e2[4], w, sth, cth;
+                fluid_tetrad(m, K, pl.u, pl.b, e1, e2, w, sth, cth);
+                float xn[4];
+                sur_features_r<R>(pl.Te, pl.B, w * nu_obs, sth, cth, R(p.model.kappa), f);
 #pragma unroll
-            for (int j = 0; j < 4; j++) xn[j] = 2.0f * (f[j] - p.sur_lo[j]) / (p.sur_hi[j] - p.sur_lo[j]) - 1.0f;
-            o = make_float4(xn[0], xn[1], xn[2], xn[3]);
+                for (int j = 0; j < 4; j++) xn[j] = 2.0f * (f[j] - p.sur_lo[j]) / (p.sur_hi[j] - p.sur_lo[j]) - 1.0f;
+                o = make_float4(xn[0], xn[1], xn[2], xn[3]);
+            }
+            if (p.sur_row) {
+                p.feat[row + base + lane] = o;
+                p.sur_row[st] = (int)(row + base + lane);
+            } else if (p.feat) {
+                p.feat[st] = o;
+            }
         }
-        if (p.sur_row) {
-            p.feat[row + n] = o;
-            p.sur_row[(long long)blk * kBlockStates + slot] = (int)(row + n);
-        } else if (p.feat) {
-            p.feat[(long long)blk * kBlockStates + slot] = o;
+        if (p.feat_raw) {  // one counter update a warp
+            const unsigned em = __ballot_sync(full, valid);
+            unsigned long long k = 0;
+            if (lane == 0 && em) k = atomicAdd(&p.ctr->feat_count, (unsigned long long)__popc(em));
+            k = __shfl_sync(full, k, 0) + __popc(em & ((1u << lane) - 1u));
+            if (valid && (long long)k < p.feat_cap) p.feat_raw[k] = make_float4(f[0], f[1], f[2], f[3]);
         }
-        if (n == 0) live = false;
+        blk = prev;
+        base -= kBlockStates;
     }
 }
 

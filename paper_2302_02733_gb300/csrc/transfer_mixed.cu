@@ -43,7 +43,7 @@ void launch_unpol(const XferArgs &a, int grid, cudaStream_t s) {
         unpol_kernel<float><<<grid, kXferThreads, 0, s>>>(a);
 }
 void launch_sur_features(const XferArgs &a, int grid, cudaStream_t s) {
-    grid = ray_grid(grid, a.nrays, kXferThreads);
+    grid = ray_grid(grid, a.nrays, kXferThreads / 32);
     sur_features_pass<float><<<grid, kXferThreads, 0, s>>>(a);
 }
 static int func_regs(const void *f) {
