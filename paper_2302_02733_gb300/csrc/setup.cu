@@ -3,19 +3,9 @@
 
 namespace prt {
 
-// theta at X2 and blend weight w
-__device__ __forceinline__ double fmks_theta(const GridModel &g, double w, double x2) {
-    double s, c;
-    const double y = x2 - 0.5, yp = 2.0 * y;
-    sincos(2.0 * kPi * y, &s, &c);
-    const double mug = kPi * y - 0.5 * (1.0 - g.hslope) * s, ya = pow(fabs(yp / g.poly_xt), g.poly_alpha);
-    const double muj = g.poly_norm * yp * (1.0 + ya / (g.poly_alpha + 1.0));
-    return 0.5 * kPi + (mug + w * (muj - mug));
-}
-
 // Table of X2(w, theta) for the FMKS map theta = theta_G(X2) + w (theta_J(X2) - theta_G(X2)),
 // w in [0, 1] (64 rows), theta in [0, pi] (1024 columns), by bisection to the last bit. The
-// transfer kernels' inverse (polarmap.cuh) starts from a bilinear read of this table.
+// transfer kernels start Newton's method from a bilinear read of this table.
 __global__ void x2_table_kernel(GridModel g, double *tab, float *tabf) {
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= kX2TabW * kX2TabT) return;
@@ -25,7 +15,7 @@ __global__ void x2_table_kernel(GridModel g, double *tab, float *tabf) {
     double lo = 0.0, hi = 1.0;
     for (int k = 0; k < 70; k++) {
         double mid = 0.5 * (lo + hi);
-        if (fmks_theta(g, w, mid) < th)
+        if (fmks_theta_w<double>(g, w, mid, nullptr, nullptr) < th)
             lo = mid;
         else
             hi = mid;

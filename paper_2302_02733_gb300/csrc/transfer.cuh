@@ -635,6 +635,63 @@ __device__ __forceinline__ void adaf_plasma(const AdafModel &p, R a, const KS<R>
     o.valid = true;
 }
 
+// FMKS polar angle in offset form: mu = theta - pi/2 as a function of y = X2 - 1/2, at blend
+// weight w = exp(s (X1_in - X1)); also d theta / d X2 and theta_j - theta_g. With x2 = 1/2 + y,
+// sin(2 pi x2) = -sin(2 pi y) and cos(2 pi x2) = -cos(2 pi y), so every term is small near the
+// equator and an FP32 evaluation keeps the relative precision of mu there.
+template <typename R>
+__device__ __forceinline__ R fmks_mu(const GridModel &g, R w, R y, R *dth2, R *thj_m_thg) {
+    typedef Mth<R> F;
+    R s2p, c2p;
+    F::sincos_(R(2 * kPi) * y, &s2p, &c2p);
+    R omh = R(1) - pick<R>(g.hslope, g.f_hslope);
+    R mug = R(kPi) * y - R(0.5) * omh * s2p;  // theta_g - pi/2
+    R dthg = R(kPi) * (R(1) - omh * c2p);
+    R yp = R(2) * y;                          // 2 X2 - 1
+    R yx = yp / pick<R>(g.poly_xt, g.f_poly_xt);
+    R ya = F::pow_(fabs(yx), pick<R>(g.poly_alpha, g.f_poly_alpha));
+    R N = pick<R>(g.poly_norm, g.f_poly_norm);
+    R muj = N * yp * (R(1) + ya / pick<R>(g.poly_alpha + 1.0, g.f_poly_alpha1));  // theta_j - pi/2
+    R dthj = R(2) * N * (R(1) + ya);
+    if (dth2) *dth2 = dthg + w * (dthj - dthg);
+    if (thj_m_thg) *thj_m_thg = muj - mug;
+    return mug + w * (muj - mug);
+}
+
+// FMKS polar angle theta(X2) at blend weight w, and d/dX2.
+template <typename R>
+__device__ __forceinline__ R fmks_theta_w(const GridModel &g, R w, R x2, R *dth2, R *thj_m_thg) {
+    return R(0.5 * kPi) + fmks_mu(g, w, x2 - R(0.5), dth2, thj_m_thg);
+}
+
+// y = X2 - 1/2 of the point at polar angle th (mu = th - pi/2, formed before rounding to FP32):
+// a table guess in (w, theta), then Newton on mu.
+__device__ __forceinline__ float fmks_y(const GridModel &g, float w, float th, float mu) {
+    float fw = w * float(kX2TabW - 1);
+    float ft = th * float((kX2TabT - 1) / kPi);
+    // fw in [0, 63], ft in [0, 1023]: no conversion instructions
+    int iw = min(max(floor_small(fw), 0), kX2TabW - 2);
+    int it = min(max(floor_small(ft), 0), kX2TabT - 2);
+    float tw = fw - i2f_small(iw);
+    float tt = ft - i2f_small(it);
+    const float *T = g.x2_table_f;
+    float x00 = T[iw * kX2TabT + it], x01 = T[iw * kX2TabT + it + 1];
+    float x10 = T[(iw + 1) * kX2TabT + it], x11 = T[(iw + 1) * kX2TabT + it + 1];
+    float y = (1.0f - tw) * ((1.0f - tt) * x00 + tt * x01) + tw * ((1.0f - tt) * x10 + tt * x11) - 0.5f;
+    // the bilinear table guess is within 1.3e-5 of the root in y (a cell is 1/n2 = 7.8e-3); one
+    // Newton step takes that below 1e-9. Two all the same: after one the result still depends on how
+    // the guess was rounded, which differs between the kernels this is inlined into (the single,
+    // batched and staged transfers give bit-identical mixed images only after the second)
+    const int iters = 2;
+#pragma unroll
+    for (int k = 0; k < iters; k++) {
+        float d;
+        float f = fmks_mu(g, w, y, &d, (float *)nullptr) - mu;
+        y -= f / d;
+    }
+    return fmin(fmax(y, -0.5f), 0.5f);
+}
+
 // Corner index and fraction of one axis of the trilinear fetch, from an approximate cell
 // coordinate (within one cell of the truth) and the exact fraction relative to that corner;
 // clamped to the first and last cell centres.
@@ -666,7 +723,7 @@ struct GridCell {
     int i0, j0, k0, k1;
     R r, w, y;      // r in R, the FMKS blend weight and y = X2 - 1/2
     R w1, w2, w3;   // trilinear fractions
-    R dth2, dd;     // d theta / d X2 and theta_j - theta_g
+    R dth2, dd;     // FP64: d theta / d X2 and theta_j - theta_g
 };
 
 // false outside r_in <= r <= r_out
@@ -694,7 +751,7 @@ __device__ __forceinline__ bool grid_cell(const GridModel &g, double rd, double 
         w1 = log1pf(dl) / g.f_dx1;  // ln(r / r_c) / dx1
         cell_axis(g.n1, i0, w1);
         // theta - pi/2 from the pair, pi/2 = 1.57079637f - 4.37113883e-8f
-        y = fmks_y32(g, w, th, (th - 1.57079637f) + (thl + 4.37113883e-8f), c.dth2, c.dd);
+        y = fmks_y(g, w, th, (th - 1.57079637f) + (thl + 4.37113883e-8f));
         float t = y * i2f_small(g.n2), c2 = 0.5f * i2f_small(g.n2 - 1);
         j0 = min(max(floor_small(t + c2), 0), g.n2 - 2);
         w2 = t - (i2f_small(j0) - c2);
@@ -795,7 +852,8 @@ __device__ __forceinline__ void grid_state(const GridModel &g, const KS<R> &m, c
     const R r = c.r;
     R rho = P[0], uu = P[1];
     if (!(rho > R(0)) || !(uu > R(0))) return;
-    const R dth2 = c.dth2, dd = c.dd;
+    R dth2 = c.dth2, dd = c.dd;
+    if (sizeof(R) == 4) fmks_mu(g, c.w, c.y, &dth2, &dd);
     R dth1 = -pick<R>(g.mks_smooth, g.f_mks_smooth) * c.w * dd;
     R Ut[4] = {R(0), r * P[2], dth1 * P[2] + dth2 * P[3], P[4]};
     R Bi[4] = {R(0), r * P[5], dth1 * P[5] + dth2 * P[6], P[7]};

@@ -1164,7 +1164,7 @@ __global__ void __launch_bounds__(kXferThreads, 5) sur_features_pass(XferArgs p)
 // block's emitting states then follow one another, every lane adding the value that the state's lane
 // holds (11 instructions a state). With one lane per ray the states of a ray were a serial chain of a
 // point's whole evaluation each, and 16,384 rays filled a ninth of the chip: a torus at 128^2 took
-// 7.1 ms, then 0.78, at 1024^2 34.8, before fmks_y32 (256 threads and 3 blocks, with or without a barrier per block of
+// 7.1 ms, now 0.78, at 1024^2 34.8 (256 threads and 3 blocks, with or without a barrier per block of
 // states, 34.7 and 36.0; 128 threads and 4 blocks 39.8).
 template <typename R, bool JOBS = false>
 __global__ void __launch_bounds__(kXferThreads, 6) unpol_kernel(XferArgs p) {

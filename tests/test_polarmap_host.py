@@ -8,8 +8,6 @@ and ya = |2 y / xt|^alpha (relative error (alpha |ln| + 3) eps, once for the tab
   leaves out;
 - slope: eps times 16 of its terms, 4 N ya (alpha |ln| + 3) eps, the slope's change over the error of y,
   and the Taylor remainder, below 1e-16 |alpha - 3| f1 / |y| + 1e-15 as the step's own is below 1e-16 f1.
-The FP32 form likewise with eps = 2^-24: ya is off by alpha / 2 of its division's and 4 of the power's
-roundings, y by two of its own, and the step and the series leave out 1e-9 f1 and 1e-8 |alpha - 3| f1 / |y|.
 No GPU is used."""
 import os
 import shutil
@@ -38,26 +36,10 @@ namespace prt {
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kX2TabW = 64, kX2TabT = 1024;
 }
-static void sincospif(float x, float *s, float *c) {
-    const long double p = 3.14159265358979323846264338327950288L * x;
-    *s = (float)sinl(p), *c = (float)cosl(p);
-}
-static float __fmaf_rn(float a, float b, float c) { return fmaf(a, b, c); }
-static float __fmul_rn(float a, float b) { return a * b; }
-static float __fadd_rn(float a, float b) { return a + b; }
-static float __fdiv_rn(float a, float b) { return a / b; }
-static float __fdividef(float a, float b) { return a / b; }
-static int floor_small(float x) { return (int)floorf(x); }
-static float i2f_small(int i) { return (float)i; }
 #include "polarmap.cuh"
 using namespace prt;
 typedef long double L;
-struct G {
-    double hslope, poly_xt, poly_alpha, poly_norm;
-    const double *x2_table;
-    float f_hslope, f_poly_xt, f_poly_alpha, f_poly_alpha1, f_poly_norm;
-    const float *x2_table_f;
-};
+struct G { double hslope, poly_xt, poly_alpha, poly_norm; const double *x2_table; };
 static const L PI = 3.14159265358979323846264338327950288L;
 static void map(const G &g, L w, L y, L &mu, L &f1, L &dd, L &f2, L &ya) {
     const L s = sinl(2 * PI * y), c = cosl(2 * PI * y), o = 1 - (L)g.hslope, N = g.poly_norm, al = g.poly_alpha;
@@ -70,7 +52,7 @@ static void map(const G &g, L w, L y, L &mu, L &f1, L &dd, L &f2, L &ya) {
     f2 = g2 + w * (y != 0 ? 2 * N * ya * al / y - g2 : 0);
 }
 int main(int, char **v) {
-    G g, gf;
+    G g;
     g.poly_xt = atof(v[1]), g.poly_alpha = atof(v[2]), g.hslope = atof(v[3]);
     g.poly_norm = 0.5 * kPi / (1.0 + 1.0 / ((g.poly_alpha + 1.0) * std::pow(g.poly_xt, g.poly_alpha)));
     std::vector<double> tab(kX2TabW * kX2TabT);
@@ -86,13 +68,6 @@ int main(int, char **v) {
         tab[i] = 0.5 + (lo + hi) / 2;
     }
     g.x2_table = tab.data();
-    // the FP32 form's parameters, and the map with those values
-    std::vector<float> tabf(tab.begin(), tab.end());
-    gf = g;
-    gf.x2_table_f = tabf.data();
-    gf.f_poly_xt = (float)g.poly_xt, gf.f_poly_alpha = (float)g.poly_alpha, gf.f_hslope = (float)g.hslope;
-    gf.f_poly_norm = (float)g.poly_norm, gf.f_poly_alpha1 = (float)(g.poly_alpha + 1.0);
-    gf.poly_xt = gf.f_poly_xt, gf.poly_alpha = gf.f_poly_alpha, gf.hslope = gf.f_hslope, gf.poly_norm = gf.f_poly_norm;
     long n = 0, bad = 0;
     const L eps = ldexpl(1, -53);
     for (int a = 0; a <= 40; a++)
@@ -111,20 +86,6 @@ int main(int, char **v) {
             if (!(fabsl(m - mu) <= e0 && fabsl(d1 - f1) <= e1 && fabsl(d0 - dd) <= e2) && bad++ < 10)
                 std::printf("w %.4f mu %.6e y %.6e: mu off %.2Le of %.2Le, slope %.2Le of %.2Le, dd %.2Le of %.2Le\n", w, mu, y,
                             fabsl(m - mu), e0, fabsl(d1 - f1), e1, fabsl(d0 - dd), e2);
-            {
-                const float mf = (float)mu, wf = (float)w;
-                float h1, h0;
-                const float yf = fmks_y32(gf, wf, mf + 1.57079637f, mf, h1, h0);
-                map(gf, wf, yf, m, f1, dd, f2, ya);
-                const L ep = ldexpl(1, -24), al = gf.poly_alpha, Nf = gf.poly_norm, af = std::max(std::fabs(yf), 1e-30f);
-                const L e0 = ep * (8 * PI + 4 * f1 + 4 * Nf * af * ya * (al + 8)) + 1e-9L * f1;
-                const L e1 = ep * (16 * (2 * PI + 2 * Nf * (1 + ya)) + 4 * Nf * ya * (al + 8)) + fabsl(f2) * e0 / f1 +
-                             1e-8L * fabsl(al - 3) * f1 / af;
-                const L e2 = e0 + ep * 16 * PI + (f1 + 2 * Nf * (1 + ya) + 2 * PI) * e0 / f1 + e1 * 1e-3L;
-                if (!(fabsl(m - mf) <= e0 && fabsl(h1 - f1) <= e1 && fabsl(h0 - dd) <= e2) && bad++ < 10)
-                    std::printf("FP32 w %.4f mu %.6e y %.6e: mu off %.2Le of %.2Le, slope %.2Le of %.2Le, dd %.2Le of %.2Le\n", w,
-                                mu, (double)yf, fabsl(m - mf), e0, fabsl(h1 - f1), e1, fabsl(h0 - dd), e2);
-            }
         }
     std::printf("points %ld failures %ld\n", n, bad);
     return bad != 0;
