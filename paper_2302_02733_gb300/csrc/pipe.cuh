@@ -207,7 +207,7 @@ __device__ __forceinline__ void pipe_geodesic(const PipeArgs &p, const GeoTabs &
 }
 
 template <typename R, typename OutT>
-__device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *tab) {
+__device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *sgw) {
     long long ray = -1;
     int job = 0, blk = -1, slot = 0, n = 0, rstat = 0;
     unsigned long long ticket = 0, wait_t0 = 0;
@@ -282,7 +282,7 @@ __device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *tab) {
         const double4_32a *src = reinterpret_cast<const double4_32a *>(p.pool.states + (long long)blk * kBlockStates + slot);
         double4_32a q0 = load_cg(src), q1 = load_cg(src + 1);
         KS<R> m;
-        if (xfer_point(J.cam, J.model, q0, q1, tab, Ln, m)) my_emit++;
+        if (xfer_point(J.cam, J.model, q0, q1, sgw, Ln, m)) my_emit++;
         my_pts++;
         if (n == 0) {
             int ix, iy;
@@ -303,14 +303,15 @@ __device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *tab) {
 
 template <typename R, typename OutT>
 __global__ void __launch_bounds__(kPipeThreads, sizeof(R) == 4 ? 2 : 1) pipe_kernel(PipeArgs p) {
+    __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
     __shared__ __align__(16) fx64 fxtab[2 * kFxTab];  // the geodesic's sin/cos table
-    const R *tab = thermal_tab<R>(p.therm);
+    const R *sgw = thermal_weights(wsh, p.therm);
     load_fx_table(p.sctab, fxtab);
     __syncthreads();
     if ((int)(threadIdx.x >> 5) < ((blockIdx.x & 1) ? p.geo_warps_odd : p.geo_warps))
         pipe_geodesic(p, GeoTabs{fxtab, p.sctab});
     else
-        pipe_transfer<R, OutT>(p, tab);
+        pipe_transfer<R, OutT>(p, sgw);
 }
 
 }  // namespace prt

@@ -38,7 +38,7 @@ struct rt_ctx {
     double *d_stats = nullptr;
     double *d_sctab = nullptr;  // the geodesic's sin and cos tables
     double *d_kap = nullptr;    // tables of the kappa quadrature
-    double *d_therm = nullptr;  // tables of the thermal rotativities
+    double *d_therm = nullptr;  // FP64 tables of the thermal rotativities
     // surrogate MLP: parameters | Adam m | Adam v | gradient (FP32), tensor-core images, scalars
     float *d_theta = nullptr;
     void *d_wpk = nullptr, *d_tpk = nullptr, *d_mlpaux = nullptr;

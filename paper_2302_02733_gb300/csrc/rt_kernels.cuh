@@ -99,7 +99,7 @@ struct XferArgs {
     const int *pix_list;  // optional: the pixel of each global ray id (adaptive rendering)
     const JobDev *jobs;   // optional: a table of images (see GeoArgs)
     int njobs;
-    const double *therm;  // the thermal tables (ThermTab, ThermTabF)
+    const double *therm;  // FP64: the thermal tables (ThermTab)
     double *ext;          // FP64: 4 doubles per saved state for the points' records, or NULL (then one
                           // kernel does the whole transfer)
 };
@@ -169,7 +169,7 @@ struct PipeArgs {
     int geo_warps;      // 1..7
     int step_tile;      // RK4 steps per lane between queue and pool checks
     int geo_warps_odd;  // 1..7: the geodesic warps of odd-numbered blocks
-    const double *therm;  // the thermal tables (ThermTab, ThermTabF)
+    const double *therm;  // FP64: the thermal tables (ThermTab)
 };
 
 void launch_pool_init(const Pool &p, PipeCounters *c, cudaStream_t s);
@@ -178,8 +178,8 @@ void launch_pipe_mixed(const PipeArgs &a, int grid, cudaStream_t s);
 int pipe_blocks_per_sm_fp64();
 int pipe_blocks_per_sm_mixed();
 
-// Tables of the thermal rotativities (ThermTab and ThermTabF, transfer.cuh)
-constexpr size_t kThermTabBytes = (960 * 18 + 704 * 20) * sizeof(double) + (80 + 44) * 32 * 8 * sizeof(float);
+// FP64 tables of the thermal rotativities (ThermTab, transfer.cuh)
+constexpr size_t kThermTabBytes = (960 * 18 + 704 * 20) * sizeof(double);
 int launch_thermal_tables(double *buf, cudaStream_t s);
 
 // ---- kappa-distribution coefficients by quadrature (kappa.cuh) ---------------------------

@@ -82,44 +82,6 @@ __global__ void therm_table_kernel(double *tab, int e0, int n) {
     for (int q = 0; q <= D; q++) tab[(2 * i + j) * (D + 1) + q] = ldexp(p[q], q);
 }
 
-// The FP32 tables of ThermTabF, one thread a segment: Chebyshev fits of degree D, as powers of u.
-template <int D, void (*fn)(double, double *)>
-__device__ void therm_powers(double lo, double width, int which, float *out) {
-    double f[D + 1], p[D + 1], a[D + 1], b[D + 1];
-    for (int j = 0; j <= D; j++) {
-        double v[2];
-        fn(lo + width * (0.5 + 0.5 * cospi((j + 0.5) / (D + 1))), v);
-        f[j] = v[which];
-        p[j] = 0.0, a[j] = j == 0, b[j] = j == 1;
-    }
-    for (int k = 0; k <= D; k++) {
-        double s = 0.0, c[D + 1];
-        for (int q = 0; q <= D; q++) s += f[q] * cospi(k * (q + 0.5) / (D + 1));
-        s *= (k == 0 ? 1.0 : 2.0) / (D + 1);
-        for (int q = 0; q <= D; q++) {
-            p[q] += s * a[q];
-            c[q] = (q > 0 ? 2.0 * b[q - 1] : 0.0) - a[q];
-        }
-        for (int q = 0; q <= D; q++) a[q] = b[q], b[q] = c[q];
-    }
-    for (int q = 0; q <= D; q++) out[q] = (float)ldexp(p[q], q);
-}
-__global__ void therm_table_f_kernel(float *tab) {
-    typedef ThermTabF T;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T::nb + T::ns) return;
-    const int k = i < T::nb ? i : i - T::nb, e0 = i < T::nb ? T::eb : T::es;
-    const double oct = ldexp(1.0, e0 + (k >> 5)), lo = oct * (1.0 + (k & 31) / 32.0), width = oct / 32.0;
-    float *o = tab + (i < T::nb ? 0 : T::shc) + 8 * k;
-    if (i < T::nb) {
-        therm_powers<3, bessel_ratio_values>(lo, width, 0, o);
-        therm_powers<3, bessel_ratio_values>(lo, width, 1, o + 4);
-    } else {
-        therm_powers<4, shcherbakov_values>(lo, width, 0, o);
-        therm_powers<2, shcherbakov_values>(lo, width, 1, o + 5);
-    }
-}
-
 int launch_thermal_tables(double *buf, cudaStream_t s) {
     typedef ThermTab T;
     static_assert(T::nb % kThermPerBlock == 0 && T::ns % kThermPerBlock == 0, "whole blocks");
@@ -127,7 +89,6 @@ int launch_thermal_tables(double *buf, cudaStream_t s) {
         <<<T::nb / kThermPerBlock, kThermPerBlock * (T::db + 1), 0, s>>>(buf + T::bes, T::eb, T::nb);
     therm_table_kernel<T::ds, shcherbakov_values>
         <<<T::ns / kThermPerBlock, kThermPerBlock * (T::ds + 1), 0, s>>>(buf + T::shc, T::es, T::ns);
-    therm_table_f_kernel<<<(ThermTabF::nb + ThermTabF::ns + 63) / 64, 64, 0, s>>>(reinterpret_cast<float *>(buf + T::size));
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

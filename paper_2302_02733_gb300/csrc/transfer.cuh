@@ -73,11 +73,22 @@ struct Mth<float> {
 };
 
 // ------------------------------------------------------------------------------------------
-// e^z K_n(z), n = 0, 1, 2, by ascending series (Abramowitz & Stegun 9.6.11, 9.6.13) for z < 2; in FP64
-// above Theta = 2^20, where the tables end:
-//   K0 = -(ln(z/2) + gamma) I0 + sum H_k t^k/(k!)^2,
-//   K1 = 1/z + (ln(z/2) + gamma) I1 - (z/4) sum (H_k + H_{k+1}) t^k/(k!(k+1)!),  t = z^2/4,
-//   K2 = K0 + (2/z) K1.
+// e^z K_n(z), n = 0, 1, 2.
+//   z < 2: ascending series (Abramowitz & Stegun 9.6.11, 9.6.13),
+//     K0 = -(ln(z/2) + gamma) I0 + sum H_k t^k/(k!)^2,
+//     K1 = 1/z + (ln(z/2) + gamma) I1 - (z/4) sum (H_k + H_{k+1}) t^k/(k!(k+1)!),  t = z^2/4;
+//   z >= 2: with u = sqrt(2z) sinh(s/2) in K_n = int_0^inf e^{-z cosh s} cosh(ns) ds,
+//     e^z K_n(z) = sqrt(2/z) int_0^inf e^{-u^2} c_n(u) / sqrt(1 + u^2/(2z)) du,
+//     c_0 = 1, c_1 = 1 + u^2/z, c_2 = 2 c_1^2 - 1, by the trapezoid rule on fixed nodes u_k = k h
+//     (the integrand is analytic in |Im u| < sqrt(2z), so the rule converges geometrically).
+//   K2 = K0 + (2/z) K1 for the series branch.
+// In FP32 on every call; in FP64 only above the tables' end.
+struct BesselCfg {
+    static constexpr int nser = 8, nq = 10;
+    static constexpr float h = 0.5f;
+};
+
+// The series branch in FP64 (z < 2): above Theta = 2^20, where the tables end.
 __device__ __forceinline__ void bessel_k012_series(double z, double &k0, double &k1, double &k2) {
     const double iz = 1.0 / z, hz = 0.5 * z, t = hz * hz, lg = log(hz) + 0.57721566490153286061;
     double i0 = 0, s0 = 0, i1s = 0, s1 = 0, term0 = 1, term1 = 1, H = 0;
@@ -95,6 +106,53 @@ __device__ __forceinline__ void bessel_k012_series(double z, double &k0, double 
     k0 = (s0 - lg * i0) * e;
     k1 = (iz + lg * (hz * i1s) - 0.25 * z * s1) * e;
     k2 = k0 + 2.0 * iz * k1;
+}
+
+// gw[k] = exp(-(k h)^2), halved at k = 0 (trapezoid end weight); kept in shared memory.
+__device__ __forceinline__ void bessel_k012_scaled(float z, const float *gw, float &k0, float &k1, float &k2) {
+    typedef float R;
+    typedef Mth<R> F;
+    typedef BesselCfg B;
+    R iz = R(1) / z;
+    if (z < R(2)) {
+        R hz = R(0.5) * z, t = hz * hz;
+        R lg = F::log_(hz) + R(0.57721566490153286061);
+        R i0 = 0, s0 = 0, i1s = 0, s1 = 0, term0 = 1, term1 = 1, H = 0;
+#pragma unroll
+        for (int k = 0; k < B::nser; k++) {
+            R ik1 = R(1) / R(k + 1);
+            i0 += term0;
+            s0 += H * term0;
+            i1s += term1;
+            s1 += (R(2) * H + ik1) * term1;
+            H += ik1;
+            term0 *= t * ik1 * ik1;
+            term1 *= t * ik1 / R(k + 2);
+        }
+        R e = F::exp_(z);
+        R K0 = -lg * i0 + s0;
+        R K1 = iz + lg * (hz * i1s) - R(0.25) * z * s1;
+        k0 = K0 * e;
+        k1 = K1 * e;
+        k2 = k0 + R(2) * iz * k1;
+    } else {
+        R i2z = R(0.5) * iz;
+        R a0 = 0, a1 = 0, a2 = 0;
+#pragma unroll
+        for (int k = 0; k < B::nq; k++) {
+            R u = R(k) * B::h, u2 = u * u;
+            R w = gw[k];
+            R rr = w * F::rsqrt_(R(1) + u2 * i2z);
+            R c1 = R(1) + u2 * iz;
+            a0 += rr;
+            a1 += rr * c1;
+            a2 += rr * (R(2) * c1 * c1 - R(1));
+        }
+        R sc = F::sqrt_(R(2) * iz) * B::h;
+        k0 = sc * a0;
+        k1 = sc * a1;
+        k2 = sc * a2;
+    }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -133,6 +191,7 @@ struct ThermTab {
     static constexpr int eb = -40, nb = 60 * 16, es = -30, ns = 44 * 16;  // first octave, segments
     static constexpr int bes = 0, shc = nb * 2 * (db + 1), size = shc + ns * 2 * (ds + 1);
 };
+static_assert(kThermTabBytes == ThermTab::size * sizeof(double), "thermal tables' size");
 
 // The segment of v >= 2^e0 and its variable u.
 __device__ __forceinline__ int therm_segment(double v, int e0, double &u) {
@@ -151,85 +210,41 @@ __device__ __forceinline__ void therm_eval(const double *t, double u, double &a,
     }
 }
 
-// The same functions' tables for the FP32 transfer, after the FP64 ones: 32 segments an octave, eight
-// coefficients a segment (two 16-byte loads), a cubic each for the ratios, a quartic for f and a parabola
-// for g (within 3e-8, 4e-8 and 9e-8 of their values, before rounding to FP32, over the whole range). They
-// replace 10 quadrature nodes or 8 series terms (with a warp's lanes on both sides of z = 2, both) and
-// the 11 transcendental functions: the FP32 transfer of a torus at 1024^2 takes 57.6 ms instead of
-// 61.0, of an ADAF at 700^2 14.8 instead of 16.1.
-struct ThermTabF {
-    static constexpr int eb = -40, nb = 80 * 32, es = -30, ns = 44 * 32;
-    static constexpr int shc = nb * 8, size = shc + ns * 8;
-};
-static_assert(kThermTabBytes == ThermTab::size * sizeof(double) + ThermTabF::size * sizeof(float) &&
-                  ThermTab::size % 2 == 0,
-              "thermal tables' size");
-
-__device__ __forceinline__ int therm_segment(float v, int e0, float &u) {
-    const unsigned b = __float_as_uint(v);
-    u = __uint_as_float((b << 5 & 0x007fffffu) | 0x3f800000u) - 1.5f;
-    return (int)(b >> 18) - ((127 + e0) << 5);
-}
-
-// The tables that the transfer in precision R reads.
+// Ratios K0/K2 and K1/K2 at 1/Theta. gw: in FP32 the quadrature's weights, in FP64 the tables.
 template <typename R>
-__device__ __forceinline__ const R *thermal_tab(const double *t) {
-    if constexpr (sizeof(R) == 8)
-        return t;
-    else
-        return reinterpret_cast<const float *>(t + ThermTab::size);
-}
-
-// Ratios K0/K2 and K1/K2 at 1/Theta.
-__device__ __forceinline__ void bessel_ratios(double Te, const double *tab, double &r0, double &r1) {
-    double u;
-    const int i = therm_segment(Te, ThermTab::eb, u);
-    if (i < 0) {  // K_n(z)/K_2(z) -> 1 as z -> infinity
-        r0 = r1 = 1.0;
-    } else if (i < ThermTab::nb) {
-        therm_eval<ThermTab::db>(tab + ThermTab::bes + i * 2 * (ThermTab::db + 1), u, r0, r1);
-    } else {
+__device__ __forceinline__ void bessel_ratios(R Te, const R *gw, R &r0, R &r1) {
+    if constexpr (sizeof(R) == 8) {
+        double u;
+        const int i = therm_segment(Te, ThermTab::eb, u);
+        if (i < 0) {  // K_n(z)/K_2(z) -> 1 as z -> infinity
+            r0 = r1 = 1.0;
+            return;
+        }
+        if (i < ThermTab::nb) {
+            therm_eval<ThermTab::db>(gw + ThermTab::bes + i * 2 * (ThermTab::db + 1), u, r0, r1);
+            return;
+        }
         double k0, k1, k2;
         bessel_k012_series(1.0 / Te, k0, k1, k2);
         r0 = k0 / k2;
         r1 = k1 / k2;
-    }
-}
-__device__ __forceinline__ void bessel_ratios(float Te, const float *tab, float &r0, float &r1) {
-    float u;
-    const int i = therm_segment(Te, ThermTabF::eb, u);
-    if (i < 0) {
-        r0 = r1 = 1.0f;
-    } else if (i < ThermTabF::nb) {
-        const float4 a = __ldg(reinterpret_cast<const float4 *>(tab) + 2 * i),
-                     b = __ldg(reinterpret_cast<const float4 *>(tab) + 2 * i + 1);
-        r0 = fmaf(fmaf(fmaf(a.w, u, a.z), u, a.y), u, a.x);
-        r1 = fmaf(fmaf(fmaf(b.w, u, b.z), u, b.y), u, b.x);
-    } else {  // the first terms in z = 1/Theta: what follows is z^2 ln z of them
-        const float z = 1.0f / Te;
-        r1 = 0.5f * z;
-        r0 = r1 * z * (logf(2.0f * Te) - 0.57721566f);
+    } else {
+        R k0 = R(1), k1 = R(1), k2 = R(1);  // as z -> infinity
+        if (Te > R(1e-12)) bessel_k012_scaled(R(1) / Te, gw, k0, k1, k2);
+        r0 = k0 / k2;
+        r1 = k1 / k2;
     }
 }
 
 // Shcherbakov's f(X) and g(X) = 1 - 0.11 ln(1 + 0.035 X).
 template <typename R>
-__device__ __forceinline__ void shcherbakov_fg(R X, const R *tab, R &f, R &g) {
+__device__ __forceinline__ void shcherbakov_fg(R X, const R *gw, R &f, R &g) {
     typedef Mth<R> F;
-    R u;
     if constexpr (sizeof(R) == 8) {
+        double u;
         const int i = therm_segment(X, ThermTab::es, u);
         if (i >= 0 && i < ThermTab::ns) {
-            therm_eval<ThermTab::ds>(tab + ThermTab::shc + i * 2 * (ThermTab::ds + 1), u, f, g);
-            return;
-        }
-    } else {
-        const int i = therm_segment(X, ThermTabF::es, u);
-        if (i >= 0 && i < ThermTabF::ns) {
-            const float4 *t = reinterpret_cast<const float4 *>(tab + ThermTabF::shc) + 2 * i;
-            const float4 a = __ldg(t), b = __ldg(t + 1);
-            f = fmaf(fmaf(fmaf(fmaf(b.x, u, a.w), u, a.z), u, a.y), u, a.x);
-            g = fmaf(fmaf(b.w, u, b.z), u, b.y);
+            therm_eval<ThermTab::ds>(gw + ThermTab::shc + i * 2 * (ThermTab::ds + 1), u, f, g);
             return;
         }
     }
@@ -253,7 +268,7 @@ __device__ __forceinline__ void shcherbakov_fg(R X, const R *tab, R &f, R &g) {
 // the light cone |j_P| <= j_I where the fits are used out of range.
 // out: jI jQ jV aI aQ aV rQ rV
 template <typename R>
-__device__ __forceinline__ void thermal_coeffs(R ne, R Te, R B, R nu, R sth, R cth, const R *tab, R out[8]) {
+__device__ __forceinline__ void thermal_coeffs(R ne, R Te, R B, R nu, R sth, R cth, const R *gw, R out[8]) {
     typedef Mth<R> F;
 #pragma unroll
     for (int i = 0; i < 8; i++) out[i] = R(0);
@@ -269,8 +284,8 @@ __device__ __forceinline__ void thermal_coeffs(R ne, R Te, R B, R nu, R sth, R c
     R rb = nuB / nu;
     R X = Te * F::sqrt_(R(1.4142135623730951) * sth * R(1e3) * rb);
     R r0, r1, f, gX;
-    bessel_ratios(Te, tab, r0, r1);
-    shcherbakov_fg(X, tab, f, gX);
+    bessel_ratios(Te, gw, r0, r1);
+    shcherbakov_fg(X, gw, f, gX);
     out[6] = cQ2 * ne * rb * rb / nu * sth * sth * f * (r1 + R(6) * Te);
     out[7] = R(2) * cQ2 * ne * rb / nu * cth * r0 * gX;
     if (sth < R(1e-12)) return;

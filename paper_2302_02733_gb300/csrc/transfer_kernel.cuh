@@ -202,7 +202,7 @@ struct SurPrefR {
 };
 
 template <typename R>
-__device__ __forceinline__ SurPrefR<R> sur_prefactors_r(R ne, R Te, R B, R nu, R sth, R cth, const R *tab) {
+__device__ __forceinline__ SurPrefR<R> sur_prefactors_r(R ne, R Te, R B, R nu, R sth, R cth) {
     typedef Mth<R> F;
     const R cB = R(kQe / (2.0 * kPi * kMe * kC));             // nu_B / B
     const R cQ2 = R(kQe * kQe / (kMe * kC));                  // e^2 / (m c)
@@ -216,10 +216,9 @@ __device__ __forceinline__ SurPrefR<R> sur_prefactors_r(R ne, R Te, R B, R nu, R
     p.Pa = cQ2 * ne / (R(4.0 * 1.7320508075688772) * nu * Te * Te * Te);
     p.PaV = p.Pa * cot;
     R X = Te * F::sqrt_(R(1.4142135623730951) * as * R(1e3) * rb);
-    R f, g;
-    shcherbakov_fg(X, tab, f, g);
+    R f = shcherbakov_fX(X);
     p.PrQ = cQ2 * ne * rb * rb / nu * sth * sth * f;
-    p.PrV = R(2) * cQ2 * ne * rb / nu * ac * g;
+    p.PrV = R(2) * cQ2 * ne * rb / nu * ac * (R(1) - R(0.11) * F::log1p_(R(0.035) * X));
     p.sgn = cth < R(0) ? R(-1) : R(1);
     return p;
 }
@@ -285,7 +284,7 @@ __device__ __forceinline__ void kappa_point_coeffs(const XferArgs *pa, long long
                 for (int q = 0; q < kSurBasis; q++) b += nm[16 + k * kSurBasis + q] * phi[q];
                 y[k] = b + nm[k] + nm[8 + k] * yh[k];
             }
-            sur_expand_r<R>(sur_prefactors_r<R>(pl.ne, pl.Te, pl.B, w * nu_obs, sth, cth, thermal_tab<R>(pa->therm)), y, cf);
+            sur_expand_r<R>(sur_prefactors_r<R>(pl.ne, pl.Te, pl.B, w * nu_obs, sth, cth), y, cf);
             if (!(cf[0] > F::jflush))
 #pragma unroll
                 for (int k = 0; k < 6; k++) cf[k] = R(0);
@@ -325,7 +324,7 @@ struct XPoint {
 
 template <typename R, int CM = 0, bool PRE = false>
 __device__ __forceinline__ void xfer_eval(const Camera &c, const Model &mdl, const double4_32a &q0,
-                                          const double4_32a &q1, const R *tab, XPoint<R> &P, XRec<R> &x,
+                                          const double4_32a &q1, const R *sgw, XPoint<R> &P, XRec<R> &x,
                                           const XferArgs *pa = nullptr, long long st = 0,
                                           PreFetch<R> pre = PreFetch<R>{nullptr, nullptr}) {
     const R a = pick<R>(c.a, c.f_a);
@@ -354,7 +353,7 @@ __device__ __forceinline__ void xfer_eval(const Camera &c, const Model &mdl, con
     for (int i = 0; i < 4; i++) P.e1[i] = pinned(P.e1[i]), P.e2[i] = pinned(P.e2[i]);
     R cf[8];
     if (CM == 0)
-        thermal_coeffs(pl.ne, pl.Te, pl.B, w * pick<R>(c.nu_obs, c.f_nu_obs), sth, cth, tab, cf);
+        thermal_coeffs(pl.ne, pl.Te, pl.B, w * pick<R>(c.nu_obs, c.f_nu_obs), sth, cth, sgw, cf);
     else
         kappa_point_coeffs<R, CM>(pa, st, mdl, pl, w, sth, cth, pick<R>(c.nu_obs, c.f_nu_obs), cf);
     // invariant form: S holds I/nu^3, so the step takes J/w^3 and the same M
@@ -430,12 +429,12 @@ __device__ __forceinline__ void xfer_pass(const R T0[4][4], XLegs<R> &L) {
 // state. Returns whether the point emits.
 template <typename R, int CM = 0, bool PRE = false>
 __device__ __forceinline__ bool xfer_point(const Camera &c, const Model &mdl, const double4_32a &q0,
-                                           const double4_32a &q1, const R *tab, XLane<R> &Ln, KS<R> &m,
+                                           const double4_32a &q1, const R *sgw, XLane<R> &Ln, KS<R> &m,
                                            const XferArgs *pa = nullptr, long long st = 0,
                                            PreFetch<R> pre = PreFetch<R>{nullptr, nullptr}) {
     XPoint<R> P;
     XRec<R> x;
-    xfer_eval<R, CM, PRE>(c, mdl, q0, q1, tab, P, x, pa, st, pre);
+    xfer_eval<R, CM, PRE>(c, mdl, q0, q1, sgw, P, x, pa, st, pre);
     m = P.m;
     if (!Ln.basis && !P.valid) return false;
     R T0[4][4];
@@ -551,11 +550,24 @@ __device__ __forceinline__ void xfer_zero(long long pix, void *out, void *depth)
     }
 }
 
+// What the thermal coefficients read: in FP32 the Bessel quadrature's weights exp(-(k h)^2) (halved at
+// k = 0), put into shared memory here, in FP64 the tables in global memory.
+__device__ __forceinline__ const float *thermal_weights(float *sgw, const double *) {
+    if (threadIdx.x < BesselCfg::nq) {
+        float u = float(threadIdx.x) * BesselCfg::h;
+        sgw[threadIdx.x] = expf(-u * u) * (threadIdx.x == 0 ? 0.5f : 1.0f);
+    }
+    return sgw;
+}
+__device__ __forceinline__ const double *thermal_weights(double *, const double *tab) { return tab; }
+
 // JOBS: the rays run over a table of images (p.jobs), each with its own camera, model and
 // outputs; otherwise over the one image of p.cam, p.model, p.out.
 template <typename R, typename OutT, int CM = 0, bool JOBS = false>
 __global__ void __launch_bounds__(kXferThreads, sizeof(R) == 4 ? 4 : 1) transfer_kernel(XferArgs p) {
-    const R *tab = thermal_tab<R>(p.therm);
+    __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
+    const R *sgw = thermal_weights(wsh, p.therm);
+    __syncthreads();
     long long ray = -1;
     int blk = -1, slot = 0, n = 0, rstat = 0, job = 0;
     bool live = false, drained = false;
@@ -614,7 +626,7 @@ __global__ void __launch_bounds__(kXferThreads, sizeof(R) == 4 ? 4 : 1) transfer
         KS<R> m;
         const Camera &c = JOBS ? p.jobs[job].cam : p.cam;
         const Model &mdl = JOBS ? p.jobs[job].model : p.model;
-        if (xfer_point<R, CM>(c, mdl, q0, q1, tab, Ln, m, &p, (long long)blk * kBlockStates + slot)) my_emit++;
+        if (xfer_point<R, CM>(c, mdl, q0, q1, sgw, Ln, m, &p, (long long)blk * kBlockStates + slot)) my_emit++;
         my_pts++;
         if (n == 0) {
             int ix, iy;
@@ -713,7 +725,9 @@ struct PointsCfg<double> {
 // handed down lane by lane.
 template <typename R, int CM = 0, bool JOBS = false>
 __global__ void __launch_bounds__(PointsCfg<R>::threads, PointsCfg<R>::blocks) points_kernel(XferArgs p) {
-    const R *tab = thermal_tab<R>(p.therm);
+    __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
+    const R *sgw = thermal_weights(wsh, p.therm);
+    __syncthreads();
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     unsigned long long my_pts = 0, my_emit = 0;
@@ -767,7 +781,7 @@ __global__ void __launch_bounds__(PointsCfg<R>::threads, PointsCfg<R>::blocks) p
         if (act) {
             const double4_32a *src = reinterpret_cast<const double4_32a *>(p.arena.states + st);
             const double4_32a q0 = src[0], q1 = src[1];
-            xfer_eval<R, CM>(c, mdl, q0, q1, tab, P, x, &p, st);
+            xfer_eval<R, CM>(c, mdl, q0, q1, sgw, P, x, &p, st);
             connection_T(P.m, P.K, T0);
             if (P.valid) xfer_screen(P, T0, L);
         }
@@ -951,9 +965,10 @@ __device__ __forceinline__ void grid_interp_staged(const GridCell<R> &c, const f
 template <int CM = 0>
 __global__ void __launch_bounds__(kXferThreads, 4) transfer_kernel_staged(XferArgs p, const __grid_constant__ CUtensorMap tmap) {
     typedef float R;
+    __shared__ R sgw[32];
     __shared__ __align__(128) float4 stc[kXferThreads * 16];
     __shared__ __align__(8) unsigned long long bars[kXferThreads];
-    const R *tab = thermal_tab<R>(p.therm);
+    thermal_weights(sgw, p.therm);
     const uint32_t bar = smem_u32(&bars[threadIdx.x]);
     float4 *slot_s = stc + threadIdx.x * 16;
     const uint32_t slot_a = smem_u32(slot_s);
@@ -1058,7 +1073,7 @@ __global__ void __launch_bounds__(kXferThreads, 4) transfer_kernel_staged(XferAr
         }
         KS<R> m;
         PreFetch<R> pre{cmode != 0 && !failed ? &cc : nullptr, P};
-        if (xfer_point<R, CM, true>(p.cam, p.model, q0, q1, tab, Ln, m, &p, 0, pre)) my_emit++;
+        if (xfer_point<R, CM, true>(p.cam, p.model, q0, q1, sgw, Ln, m, &p, 0, pre)) my_emit++;
         my_pts++;
         if (n == 0) {
             int ix, iy;

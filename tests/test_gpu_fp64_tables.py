@@ -1,6 +1,6 @@
-"""The thermal tables, and the FP64 transfer's fixed-length series, at the ends of their ranges, against
-the oracle (which evaluates the Bessel functions, Shcherbakov's factors and the matrix exponential by
-other means), per pixel and outside the oracle's own sensitivity mask:
+"""The FP64 transfer's tables and fixed-length series at the ends of their ranges, against the oracle
+(which evaluates the Bessel functions, Shcherbakov's factors and the matrix exponential by other
+means), per pixel and outside the oracle's own sensitivity mask:
 ADAFs whose Theta_e runs below, across and above the table of K_0/K_2 and K_1/K_2 (2^-40 .. 2^20),
 and whose X runs below, across and above that of f(X) and g(X) (2^-30 .. 2^14), with optical depths
 from none to 2e4 (series of one term up to the closed form): depths to 1e-10 of the larger of the
@@ -68,25 +68,3 @@ def test_thermal_tables(rt, ora, synth, T0, n0, beta):
     assert np.abs(dref[..., 1]).max() > 0 and err[ok].max() <= 1e-10
     serr = np.abs(img - ref).max(axis=-1) / np.maximum(ref[..., 0], 1e-8 * max(ref[..., 0].max(), 1e-300))
     assert serr[ok].max() <= 1e-9
-
-
-@pytest.mark.parametrize("T0,n0,beta", [(0.1, 1e7, 1e-10), (2e-2, 3e7, 10.0), (1e6, 1e7, 1e6), (3e11, 3e7, 10.0),
-                                        (1e13, 1e3, 10.0), (1e12, 3e7, 1e-8), (1e17, 1e3, 10.0)])
-def test_thermal_tables_fp32(rt, ora, synth, T0, n0, beta):
-    """The mixed form's tables (within 1e-7 of their functions)
-    through its Faraday depths: a state's rho_V is off by a few of FP32's roundings times its terms, and
-    by the error of the field angle's cosine, some 1e-6, where that is small: 1e-5 of a pixel at the
-    median, 1e-3 of the larger of the pixel's value and a hundredth of the image's largest."""
-    polrt, ctx = rt
-    cam = synth.Camera(incl_deg=60.0, nx=12, ny=8)
-    par = synth.AdafParams(T0=T0, n0=n0, beta=beta)
-    polrt.rt_set_camera(ctx, cam)
-    polrt.rt_set_integrator(ctx, 0.05, 20000)
-    polrt.rt_load_model(ctx, polrt.adaf_model(par))
-    img = torch.zeros((8, 12, 4), dtype=torch.float32, device="cuda")
-    dep = torch.zeros((8, 12, 2), dtype=torch.float32, device="cuda")
-    polrt.rt_render_depths(ctx, polrt.RT_MIXED, img, dep)
-    dref = ora.render_image(ora.camera(cam), ora.adaf_model(par), depth=True)[4][..., 1]
-    err = np.abs(dep[..., 1].double().cpu().numpy() - dref) / np.maximum(np.abs(dref), 1e-2 * np.abs(dref).max())
-    print(f"Faraday depth: median {np.median(err):.1e} max {err.max():.1e}")
-    assert np.median(err) <= 1e-5 and err.max() <= 1e-3
