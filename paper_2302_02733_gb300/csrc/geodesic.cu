@@ -23,9 +23,13 @@ namespace prt {
 static_assert(kGeoTabBytes == 3 * kSinTab * sizeof(double) + kFxTabBytes, "sin/cos table sizes");
 
 // JOBS: the rays run over a table of images (p.jobs), each with its own camera; otherwise over
-// the one image of p.cam.
-template <bool JOBS>
-__global__ void __launch_bounds__(kGeoThreads, 3) geodesic_kernel(GeoArgs p) {
+// the one image of p.cam. BLOCKS: the blocks per SM that its registers leave room for. At 3 (168
+// registers) the integer pipes are busy, 82 ms for 1024^2 rays against 90 at 2; a launch that does not
+// fill 2 blocks per SM is bound by the latency of a step instead, which is shorter where the step's
+// values have more registers to be scheduled in (216): 5.6 against 6.0 ms for an ADAF at 64^2, 11.6
+// against 12.3 for a torus at 128^2, 15.1 to 16.9 against 14.7 at 300^2.
+template <bool JOBS, int BLOCKS>
+__global__ void __launch_bounds__(kGeoThreads, BLOCKS) geodesic_kernel(GeoArgs p) {
     // the sin/cos table in shared memory: the RK4 stages read it at data-dependent indices, and
     // through the texture path those reads queued behind the transfer's gathers
     __shared__ __align__(16) fx64 fxtab[2 * kFxTab];
@@ -189,12 +193,21 @@ int launch_geo_tables(double *tab, cudaStream_t s) {
                : -1;
 }
 
+// The rays of 2 blocks on each of the 152 SMs: up to there every ray is resident in either variant.
+constexpr long long kGeoFewRays = 2 * 152 * kGeoThreads;
+
 void launch_geodesic(const GeoArgs &a, int grid, cudaStream_t s) {
     grid = ray_grid(grid, a.nrays, kGeoThreads);
-    if (a.jobs)
-        geodesic_kernel<true><<<grid, kGeoThreads, 0, s>>>(a);
-    else
-        geodesic_kernel<false><<<grid, kGeoThreads, 0, s>>>(a);
+    if (a.nrays <= kGeoFewRays) {
+        if (a.jobs)
+            geodesic_kernel<true, 2><<<grid, kGeoThreads, 0, s>>>(a);
+        else
+            geodesic_kernel<false, 2><<<grid, kGeoThreads, 0, s>>>(a);
+    } else if (a.jobs) {
+        geodesic_kernel<true, 3><<<grid, kGeoThreads, 0, s>>>(a);
+    } else {
+        geodesic_kernel<false, 3><<<grid, kGeoThreads, 0, s>>>(a);
+    }
 }
 
 static int func_regs(const void *f) {
@@ -207,12 +220,12 @@ static int func_regs(const void *f) {
 }
 
 int geodesic_regs() {
-    return std::max(func_regs((const void *)geodesic_kernel<false>), func_regs((const void *)geodesic_kernel<true>));
+    return std::max(func_regs((const void *)geodesic_kernel<false, 3>), func_regs((const void *)geodesic_kernel<true, 3>));
 }
 
 int geodesic_blocks_per_sm() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, geodesic_kernel<false>, kGeoThreads, 0) != cudaSuccess) n = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, geodesic_kernel<false, 3>, kGeoThreads, 0) != cudaSuccess) n = 1;
     return n > 0 ? n : 1;
 }
 
