@@ -335,9 +335,10 @@ int rt_image_visibilities(rt_ctx *ctx, const void *img, int form, int stokes, vo
  * one pass of each kernel. RT_SURROGATE overlaps when chunks >= 2 is set: streamed, each
  * transfer launch's rays go through the features pass, the network (over compact rows) and
  * the transfer in turn; in halves, per chunk (both measured slower than one pass on GB300).
- * Independently of the shape, a full render records each pixel's step count, and the next
- * render of the same camera and integrator takes its rays longest first, so that no launch ends
- * waiting for a few long photon-ring rays. The first render of a new camera of 2^18 rays or more
+ * Independently of the shape, a full render of 2^17 rays or more (RT_FP64: 2^13) records each
+ * pixel's step count, and the next render of the same camera and integrator takes its rays
+ * longest first, so that no launch ends waiting for a few long photon-ring rays (smaller images
+ * are all in flight at once and run in pixel order). The first render of a new camera of 2^18 rays or more
  * predicts the counts from a probe of one ray per 8 x 8 block; the next render rebuilds the
  * order from the counts the first one recorded. The image is the same in every shape and order
  * (every ray takes the same arithmetic); only the time differs. Shapes that exceed the
@@ -382,8 +383,8 @@ const char *rt_error_string(int code);
 
 /* The device's measured FP64 FMA rate [TFLOP/s, an FMA counting 2]: independent FMA chains on
  * every SM, timed with CUDA events over five launches after a warm-up. A measurement helper
- * (the paper has no counterpart): the benchmark reports the geodesic's FP64 fraction against it
- * beside the nominal peak. Synchronizes the device. */
+ * (the paper has no counterpart): the benchmark reports the geodesic's equivalent FP64 flops against it
+ * and the FP64 transfer's. Synchronizes the device. */
 int rt_fp64_fma_peak(int device, double *tflops);
 
 /* ---- Batched rendering (image libraries, MCMC fitting) -------------------------------------
