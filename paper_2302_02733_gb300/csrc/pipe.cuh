@@ -1,9 +1,13 @@
 // The batched form: geodesics and transfers of many images in one persistent launch.
 //
 // Each 8-warp block holds both roles of the method (the paper's Section 2.1). Its first
-// geo_warps warps integrate backward geodesics (FP64) and save the states. The remaining warps
-// walk completed paths toward the camera and do the transfer (FP64 or FP32). The roles share
-// the SM, so the FP32 transfer issues while the FP64 pipe is busy with geodesics.
+// geo_warps warps integrate backward geodesics and save the states. The remaining warps walk
+// completed paths toward the camera and do the transfer (FP64 or FP32). The roles share the SM: in
+// the FP64 form the FP64 pipe's transfer and the integer pipes' geodesic, in the mixed form two
+// roles on the same pipes. Six mixed images of 128^2 to 512^2 take 294 ms here at their best shape,
+// 196 with an FP64 geodesic, and 86 as one ray space in two kernels (mode 1, which the autotuner
+// takes); whole blocks of one role (275), the step as a call (283) and transfer warps that sleep
+// until most of their lanes have a ray (294) were no remedy.
 //
 // Flow control, all in global memory:
 //  - rays come from a queue (geo_next) over all images of the batch;
