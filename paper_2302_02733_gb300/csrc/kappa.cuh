@@ -44,7 +44,7 @@ constexpr double kSynLo = -27.631021115928547;  // ln 1e-12
 constexpr int kSynN = 274;                      // up to ln 740 = 6.6067
 constexpr double kKapLo = -9.210340371976182;   // ln 1e-4
 constexpr double kKapH = 0.025;
-constexpr int kKapN = 2000;                     // up to s = 40.8; nodes beyond are computed in place
+constexpr int kKapN = 2000;                     // up to s = 40.8; nodes below and beyond are computed in place
 
 // e^x times F, G, H at x by the trapezoid rule on int_0^inf e^{-x (cosh t - 1)} c(t) dt with
 // c = cosh(5t/3)/cosh t, cosh(2t/3), cosh(t/3) and cosh(t/3)/cosh t, at step 0.125 min(1, x^-1/2)
@@ -103,12 +103,13 @@ __device__ __forceinline__ void kappa_coeffs_quad(const KappaTables &T, double n
     if (!(ne > 0.0) || !(Te > 0.0) || !(B > 0.0) || !(nu > 0.0)) return;
     if (kappa > 0.0 && !(kappa > 3.0)) return;
     const bool thermal = kappa <= 0.0;
-    const double kw = thermal ? 1.0 : (kappa - 3.0) * Te, ikw = 1.0 / kw, kp1 = kappa + 1.0;
-    const double ite = 1.0 / Te;
+    const double Td = fmax(Te, 1e-60);  // the distribution's: below, powers of p leave the FP64 range
+    const double kw = thermal ? 1.0 : (kappa - 3.0) * Td, ikw = 1.0 / kw, kp1 = kappa + 1.0;
+    const double ite = 1.0 / Td, s0 = thermal ? ite : kp1 * ikw;  // s0: -(dln q/dg) at g = 1
     double s_hi;
     if (thermal) {
-        const double ghi = 1.0 + 800.0 * Te;
-        s_hi = 0.5 * log(ghi * ghi - 1.0);
+        const double ghi1 = 800.0 * Td;
+        s_hi = 0.5 * log(ghi1 * (ghi1 + 2.0));
     } else {
         s_hi = log((1.0 + kw) * 10.0) + fmin(45.0 / (kappa - 2.34), 600.0);
     }
@@ -127,17 +128,22 @@ __device__ __forceinline__ void kappa_coeffs_quad(const KappaTables &T, double n
     const double X = emits ? nu / (1.5 * nuB * as) : 0.0, lX = emits ? log(X) : 0.0;
     // the integrals in units of h. The first node stands for the range below it too: the integrands
     // go as p^c there, c = 3 (those of dN/dg as p, p^3 and p^5), and a sum h f_0 / (1 - e^-ch) from
-    // -infinity less the integral f_0 / c below s_lo leaves h f_0 w_c
-    const double w1 = 1.0 / (1.0 - exp(-h)) - 1.0 / h, w3 = 1.0 / (1.0 - exp(-3.0 * h)) - 1.0 / (3.0 * h),
-                 w5 = 1.0 / (1.0 - exp(-5.0 * h)) - 1.0 / (5.0 * h);
+    // -infinity less the integral f_0 / c below s_lo leaves h f_0 w_c. The momenta of cold electrons (p
+    // of sqrt(2 / s0) and above) come down to s_lo: their nodes begin at s0 p^2 = 2e-6, whatever that
+    // is, and nothing is left out below
+    const bool cold = s0 > 5e4;
+    const int k0 = cold ? (int)floor((0.5 * log(2e-6 / s0) - kKapLo) / h) : 0;
+    const double w1 = 1.0 / (1.0 - exp(-h)) - (cold ? 0.0 : 1.0 / h),
+                 w3 = 1.0 / (1.0 - exp(-3.0 * h)) - (cold ? 0.0 : 1.0 / (3.0 * h)),
+                 w5 = 1.0 / (1.0 - exp(-5.0 * h)) - (cold ? 0.0 : 1.0 / (5.0 * h));
     double nacc = 0.0, rv = 0.0, rq = 0.0, e[6] = {0, 0, 0, 0, 0, 0}, fq = 0.0;
     // for g >> kappa w all integrands are powers of p (to 1e-16 from here), and the tail has a closed form
     const double s_pow = thermal ? s_hi : 37.0 + log(1.0 + kw);
     const int K = (int)floor((fmin(s_hi, s_pow) - kKapLo) / h + 1e-9);
     bool on = emits;
-    for (int k = 0; k <= K; k++) {
+    for (int k = k0; k <= K; k++) {
         const int ik = k * stride;
-        const KapNode n = ik < kKapN ? T.node[ik] : kap_node(kKapLo + ik * kKapH);
+        const KapNode n = (unsigned)ik < (unsigned)kKapN ? T.node[ik] : kap_node(kKapLo + ik * kKapH);
         double q, slope;  // N / n up to its norm is g p q; -(dln q/dg)
         const double kg = kw + n.gm1;
         if (thermal) {
@@ -147,7 +153,7 @@ __device__ __forceinline__ void kappa_coeffs_quad(const KappaTables &T, double n
             q = exp(-kp1 * log(kg * ikw));
             slope = 0.0;
         }
-        const double f3 = k == 0 ? w3 : 1.0;
+        const double f3 = k == k0 ? w3 : 1.0;
         const double N = n.p3 * q * f3;
         nacc += N;
         rv += n.wv * q * f3;
@@ -157,8 +163,8 @@ __device__ __forceinline__ void kappa_coeffs_quad(const KappaTables &T, double n
         if (on && x < 740.0) {
             if (!thermal) slope = kp1 / kg;
             double D = (n.pg - n.p3 * slope) * q;
-            if (k == 0) {  // p, p^3 and p^5 apart: q = 1 - s0 (g - 1) + .., slope q = s0 (1 + ..)
-                const double s0 = thermal ? ite : kp1 * ikw, d1 = -s0 * n.gm1;
+            if (k == k0) {  // p, p^3 and p^5 apart: q = 1 - s0 (g - 1) + .., slope q = s0 (1 + ..)
+                const double d1 = -s0 * n.gm1;
                 D = n.pg * (w1 + d1 * w3 + ((q - 1.0) - d1) * w5) - n.p3 * s0 * (w3 + (slope * q / s0 - 1.0) * w5);
             }
             const double lx = lX - n.lg2, v = (lx - kSynLo) * 8.0;
