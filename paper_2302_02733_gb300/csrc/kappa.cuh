@@ -113,6 +113,9 @@ __device__ __forceinline__ void kappa_coeffs_quad(const KappaTables &T, double n
     } else {
         s_hi = log((1.0 + kw) * 10.0) + fmin(45.0 / (kappa - 2.34), 600.0);
     }
+    // hotter: p^3 leaves the FP64 range on the way to s_hi (and an infinite s_hi, of an infinite Theta_e or
+    // kappa, would be 2^31 nodes)
+    if (!(s_hi < 236.0)) return;
     // the step by the distribution's steepness (toward large kappa it narrows to the Maxwell-Juttner
     // one). Worst errors over Theta_e 0.1 to 10 and X to 3e5: tabulated 4e-10 below kappa = 10, 7e-13,
     // 4e-14 and 2e-15 in the others, exact 9e-16, 9e-13 (where j is 1e-30 of its scale) and 4e-15.

@@ -175,3 +175,9 @@ def test_cold_electrons(host, kappa):
         assert np.isfinite(out).all()
         rest = host((1e5, 1e-13, field(10.0, 1.0), 230e9, 1.0, 0.0))
         assert abs(out[7] - rest[7]) <= 1e-6 * abs(rest[7])
+
+
+def test_unbounded_distributions_give_zeros(host):
+    """Infinite or overflowing widths: zeros, as for other rows outside, and no endless sum."""
+    for Te, kappa in ((math.inf, 0.0), (math.inf, 4.5), (1e160, 0.0), (1e200, 4.5), (1.0, math.inf), (1e200, 1e200)):
+        assert (host((1e5, Te, 10.0, 230e9, 1.0, kappa), False) == 0.0).all(), (Te, kappa)
