@@ -195,8 +195,10 @@ __device__ __forceinline__ void kappa_coeffs_quad(const KappaTables &T, double n
             e[4] += D * K1;
             e[5] += D * K2;
             // beyond their peak the emission's terms fall off as powers of p: they end where they are
-            // below an eighth of a unit in the last place of each sum
-            if ((k & 7) == 0)
+            // below an eighth of a unit in the last place of each sum. Not above x = 1, where the kernels
+            // rise by e^x yet: the terms of cold electrons pass a peak of their own there, which may lie
+            // far above what follows it and far below the power-law tail's
+            if ((k & 7) == 0 && x < 1.0)
                 on = !(N * K0 <= 1e-17 * e[0] && N * K2 <= 1e-17 * e[2] && fabs(D * K0) <= 1e-17 * fabs(e[3]) &&
                        fabs(D * K2) <= 1e-17 * fabs(e[5]) && e[0] > 0.0);
         }

@@ -181,3 +181,12 @@ def test_unbounded_distributions_give_zeros(host):
     """Infinite or overflowing widths: zeros, as for other rows outside, and no endless sum."""
     for Te, kappa in ((math.inf, 0.0), (math.inf, 4.5), (1e160, 0.0), (1e200, 4.5), (1.0, math.inf), (1e200, 1e200)):
         assert (host((1e5, Te, 10.0, 230e9, 1.0, kappa), False) == 0.0).all(), (Te, kappa)
+
+
+@pytest.mark.parametrize("kappa", [3.1, 4.5, 8.0, 12.0])
+def test_power_law_tail_of_cold_electrons(host, kappa):
+    """Emission of the tail far above a cold distribution's own peak: the sum does not end at the first of
+    the two."""
+    for Te in (1.9e-5, 1e-6, 1e-7, 1e-8, 1e-9):
+        for X in (100.0, 600.0, 2000.0):
+            check(host, Te, X, 1.0, kappa)
