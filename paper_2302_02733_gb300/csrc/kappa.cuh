@@ -153,7 +153,10 @@ __device__ __forceinline__ void kappa_coeffs_quad(const KappaTables &T, double n
             q = exp(-n.gm1 * ite);
             slope = ite;
         } else {
-            q = exp(-kp1 * log(kg * ikw));
+            // the rounding of the quotient kg / kw is raised to the power kappa: 1e-10 of q at kappa = 1e6.
+            // Below 10 that is as small as log1p's own, and 60,000 points of kappa 3 to 8 take 6.16 ms
+            // against 6.22 (points of kappa 1e5, 21.4 ms against 22.0 with the quotient's logarithm)
+            q = exp(-kp1 * (kappa < 10.0 ? log(kg * ikw) : log1p(n.gm1 * ikw)));
             slope = 0.0;
         }
         const double f3 = k == k0 ? w3 : 1.0;

@@ -190,3 +190,11 @@ def test_power_law_tail_of_cold_electrons(host, kappa):
     for Te in (1.9e-5, 1e-6, 1e-7, 1e-8, 1e-9):
         for X in (100.0, 600.0, 2000.0):
             check(host, Te, X, 1.0, kappa)
+
+
+@pytest.mark.parametrize("kappa", [99.0, 1e3, 1e4, 1e6, 1e9])
+def test_large_kappa(host, kappa):
+    """Toward the Maxwell-Juttner limit the distribution's logarithm is kappa times a small number: no digits
+    are lost to the power. At Theta_e of 20 and above what lies below the first node is under 1e-14."""
+    for Te in (20.0, 300.0):
+        check(host, Te, 10.0, 1.0, kappa)
