@@ -178,8 +178,8 @@ void launch_pipe_mixed(const PipeArgs &a, int grid, cudaStream_t s);
 int pipe_blocks_per_sm_fp64();
 int pipe_blocks_per_sm_mixed();
 
-// FP64 tables of the thermal rotativities (ThermTab, transfer.cuh)
-constexpr size_t kThermTabBytes = (960 * 18 + 704 * 20) * sizeof(double);
+// FP64 tables of the thermal rotativities (ThermTab, thermtab.cuh)
+constexpr size_t kThermTabBytes = (960 * 18 + (704 + 128) * 20) * sizeof(double);
 int launch_thermal_tables(double *buf, cudaStream_t s);
 
 // ---- kappa-distribution coefficients by quadrature (kappa.cuh) ---------------------------

@@ -30,7 +30,7 @@ void launch_x2_table(const GridModel &g, double *table, float *table_f, cudaStre
 }
 
 // The FP64 tables of ThermTab: on each segment the functions at the D + 1 Chebyshev nodes (one thread
-// each), their Chebyshev coefficients, and from those the powers of u.
+// each), then the coefficients in u (one thread a function).
 __device__ void bessel_ratio_values(double Te, double v[2]) {
     // K_n(z) e^z = int_0^inf e^{-2 z sinh^2(t/2)} cosh(n t) dt by the trapezoid rule
     const double z = 1.0 / Te, h = 0.125 * fmin(1.0, rsqrt(z));
@@ -53,42 +53,25 @@ __device__ void shcherbakov_values(double X, double v[2]) {
 
 constexpr int kThermPerBlock = 16;
 template <int D, void (*fn)(double, double *)>
-__global__ void therm_table_kernel(double *tab, int e0, int n) {
-    __shared__ double f[2][kThermPerBlock][D + 1], ch[2][kThermPerBlock][D + 1];
+__global__ void therm_table_kernel(double *tab, int bits, int e0) {
+    __shared__ double f[2][kThermPerBlock][D + 1];
     const int li = threadIdx.x / (D + 1), j = threadIdx.x % (D + 1), i = blockIdx.x * kThermPerBlock + li;
-    const double x = cospi((j + 0.5) / (D + 1));
     double v[2];
-    fn(ldexp(1.0 + ((i & 15) + 0.5 + 0.5 * x) / 16.0, e0 + (i >> 4)), v);
+    fn(ThermTab::at(i, bits, e0, cospi((j + 0.5) / (D + 1))), v);
     f[0][li][j] = v[0];
     f[1][li][j] = v[1];
     __syncthreads();
-    for (int m = 0; m < 2; m++) {
-        double s = 0.0;
-        for (int q = 0; q <= D; q++) s += f[m][li][q] * cospi(j * (q + 0.5) / (D + 1));
-        ch[m][li][j] = s * (j == 0 ? 1.0 : 2.0) / (D + 1);
-    }
-    __syncthreads();
-    if (i >= n || j >= 2) return;
-    double p[D + 1], a[D + 1], b[D + 1];  // T_k and T_k+1 in powers of x = 2 u
-    for (int q = 0; q <= D; q++) p[q] = 0.0, a[q] = q == 0, b[q] = q == 1;
-    for (int k = 0; k <= D; k++) {
-        double c[D + 1];
-        for (int q = 0; q <= D; q++) {
-            p[q] += ch[j][li][k] * a[q];
-            c[q] = (q > 0 ? 2.0 * b[q - 1] : 0.0) - a[q];
-        }
-        for (int q = 0; q <= D; q++) a[q] = b[q], b[q] = c[q];
-    }
-    for (int q = 0; q <= D; q++) tab[(2 * i + j) * (D + 1) + q] = ldexp(p[q], q);
+    if (j < 2) therm_fit<D>(f[j][li], tab + (2 * i + j) * (D + 1));
 }
 
 int launch_thermal_tables(double *buf, cudaStream_t s) {
     typedef ThermTab T;
-    static_assert(T::nb % kThermPerBlock == 0 && T::ns % kThermPerBlock == 0, "whole blocks");
-    therm_table_kernel<T::db, bessel_ratio_values>
-        <<<T::nb / kThermPerBlock, kThermPerBlock * (T::db + 1), 0, s>>>(buf + T::bes, T::eb, T::nb);
+    constexpr int B = kThermPerBlock;
+    static_assert(T::nb % B == 0 && T::ns % B == 0 && T::nf % B == 0, "whole blocks");
+    therm_table_kernel<T::db, bessel_ratio_values><<<T::nb / B, B * (T::db + 1), 0, s>>>(buf + T::bes, 4, T::eb);
+    therm_table_kernel<T::ds, shcherbakov_values><<<T::ns / B, B * (T::ds + 1), 0, s>>>(buf + T::shc, 4, T::es);
     therm_table_kernel<T::ds, shcherbakov_values>
-        <<<T::ns / kThermPerBlock, kThermPerBlock * (T::ds + 1), 0, s>>>(buf + T::shc, T::es, T::ns);
+        <<<T::nf / B, B * (T::ds + 1), 0, s>>>(buf + T::shc + T::ns * 2 * (T::ds + 1), 6, T::ef);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

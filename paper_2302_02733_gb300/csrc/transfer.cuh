@@ -16,6 +16,7 @@
 #include "ffloat.cuh"
 #include "polarmap.cuh"
 #include "rt_kernels.cuh"
+#include "thermtab.cuh"
 
 namespace prt {
 
@@ -175,47 +176,14 @@ __device__ __forceinline__ R shcherbakov_fX(R X) {
     return f;
 }
 
-// ------------------------------------------------------------------------------------------
-// FP64 tables of functions of one positive variable: a polynomial on each sixteenth of an octave,
-// found from the exponent and the top four mantissa bits, in the rest of the mantissa (as
-// u = -1/2 .. 1/2, one FP64 instruction). Two functions to a segment, D + 1 coefficients each.
-//  - ThermTab::bes: K0/K2 and K1/K2 of z = 1/Theta for Theta from 2^-40 (1e-12) to 2^20;
-//  - ThermTab::shc: Shcherbakov's f(X) and 1 - 0.11 ln(1 + 0.035 X) for X from 2^-30 to 2^14.
-// 17 and 19 FP64 instructions in place of 27 reciprocal square roots (14 series terms at z < 2) and of
-// 11 transcendental functions; the FP64 pipe bounds the kernel. With fmks_y64 the FP64 instructions of
-// 32 states go from 1,721 to 1,343 and the points of a torus at 200^2 from 51 to 36 ms; an ADAF's
-// transfer at 64^2 from 16.4 to 9.5 ms. The functions have no singular point nearer than 16 segments,
-// so the fits converge as (1/66)^D; the values behind them are sums of positive terms.
-struct ThermTab {
-    static constexpr int db = 8, ds = 9;                    // degrees
-    static constexpr int eb = -40, nb = 60 * 16, es = -30, ns = 44 * 16;  // first octave, segments
-    static constexpr int bes = 0, shc = nb * 2 * (db + 1), size = shc + ns * 2 * (ds + 1);
-};
 static_assert(kThermTabBytes == ThermTab::size * sizeof(double), "thermal tables' size");
-
-// The segment of v >= 2^e0 and its variable u.
-__device__ __forceinline__ int therm_segment(double v, int e0, double &u) {
-    const long long b = __double_as_longlong(v);
-    u = __longlong_as_double((b << 4 & 0x000fffffffffffffll) | 0x3ff0000000000000ll) - 1.5;
-    return (int)(b >> 48) - ((1023 + e0) << 4);
-}
-template <int D>
-__device__ __forceinline__ void therm_eval(const double *t, double u, double &a, double &b) {
-    a = t[D];
-    b = t[2 * D + 1];
-#pragma unroll
-    for (int k = D - 1; k >= 0; k--) {
-        a = fma(a, u, t[k]);
-        b = fma(b, u, t[D + 1 + k]);
-    }
-}
 
 // Ratios K0/K2 and K1/K2 at 1/Theta. gw: in FP32 the quadrature's weights, in FP64 the tables.
 template <typename R>
 __device__ __forceinline__ void bessel_ratios(R Te, const R *gw, R &r0, R &r1) {
     if constexpr (sizeof(R) == 8) {
         double u;
-        const int i = therm_segment(Te, ThermTab::eb, u);
+        const int i = therm_segment(Te, 4, ThermTab::eb, u);
         if (i < 0) {  // K_n(z)/K_2(z) -> 1 as z -> infinity
             r0 = r1 = 1.0;
             return;
@@ -242,8 +210,8 @@ __device__ __forceinline__ void shcherbakov_fg(R X, const R *gw, R &f, R &g) {
     typedef Mth<R> F;
     if constexpr (sizeof(R) == 8) {
         double u;
-        const int i = therm_segment(X, ThermTab::es, u);
-        if (i >= 0 && i < ThermTab::ns) {
+        const int i = ThermTab::shc_segment(X, u);
+        if (i >= 0) {
             therm_eval<ThermTab::ds>(gw + ThermTab::shc + i * 2 * (ThermTab::ds + 1), u, f, g);
             return;
         }
