@@ -259,7 +259,8 @@ __device__ __forceinline__ unsigned fx_beyond(fx64 m, fx64 lo, fx64 hi) {
 //   Dt = (rho / 4) dq/dth 2^2g, Ap = F_ph 2^g = s J + 2 sa c v u 2^-g, F_th 2^g = F1 - sa c u P 2^(z - g).
 // Every term in 1 / sin is written with P. A negative number in bad is a bound that failed.
 __device__ __forceinline__ void fx_rates(const FxScale &S, const FxState &y, Fx<62> s, Fx<62> c, fx64 nk[4], unsigned &bad) {
-    const int e1 = S.e - 1, g = S.g, g2 = 2 * S.g, g3 = 3 * S.g;
+    // counts of 64 and more (r above 2^22) leave a sign, as 63 does
+    const int e1 = S.e - 1, g = S.g, g2 = g < 31 ? 2 * g : 63, g3 = g < 21 ? 3 * g : 63;
     // position terms
     const Fx<64> nal2 = S.nal2.over(g2);
     const Fx<60> na2s2 = nal2 * (s * s);                              // >= -1/4
@@ -308,7 +309,7 @@ __device__ __forceinline__ void fx_rates(const FxScale &S, const FxState &y, Fx<
     const Fx<60> npi{fx_shl(nA.m, 1) - (1ll << 60)};                  // -(r^2 + a^2) / Sigma
     const Fx<60> nkv = fx_dot_fine(isig, F1.up<2>(), npi, cz);
     // phi: (isig / s) (2 sa c v P 2^-g + (al s Fm + G) / 2^z)
-    const fx64 sm = s.m < (1ll << 62) ? s.m : (1ll << 62) - 1;
+    const fx64 sm = (unsigned long long)s.m < 1ull << 62 ? s.m : (1ll << 62) - 1;  // (a negative one fails below)
     const int zs = fx_clz((unsigned long long)(sm | 1)) - 2;          // s 2^zs in [1/2, 1)
     const Fx<61> isn = fx_recip<61>(Fx<60>{fx_shl(sm, zs) >> 2});
     const Fx<60> B = (scv * y.P).twice() + (G - fx_fine<1>(as, nFm)).dn<1>().over(S.z);
