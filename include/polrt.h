@@ -338,7 +338,8 @@ int rt_image_visibilities(rt_ctx *ctx, const void *img, int form, int stokes, vo
  * Independently of the shape, a full render of 2^17 rays or more (RT_FP64: 2^13) records each
  * pixel's step count, and the next render of the same camera and integrator takes its rays
  * longest first, so that no launch ends waiting for a few long photon-ring rays (smaller images
- * are all in flight at once and run in pixel order). The first render of a new camera of 2^18 rays or more
+ * are all in flight at once and run in pixel order, unless they are rendered in parts: overlapped,
+ * or in chunks of a small workspace, which the order gives equal shares of long rays). The first render of a new camera of 2^18 rays or more
  * predicts the counts from a probe of one ray per 8 x 8 block; the next render rebuilds the
  * order from the counts the first one recorded. The image is the same in every shape and order
  * (every ray takes the same arithmetic); only the time differs. Shapes that exceed the

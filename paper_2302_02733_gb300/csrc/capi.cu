@@ -27,7 +27,7 @@ constexpr int kAutoLastDiv = 1;
 // automatic streamed shape: about 2^kStreamChunkShift rays per chunk, at least 16 per piece, the
 // geodesic at its own occupancy
 constexpr int kStreamChunkShift = 15;
-// Images of fewer rays run in pixel order: they fill the lanes at most about twice, and a warp of
+// Images of fewer rays in one part run in pixel order: they fill the lanes at most about twice, and a warp of
 // only long rays takes longer a step than one whose lanes are leaving (geodesics, pixel order
 // against longest first: 64^2 5.4 / 6.3 ms, 128^2 6.4 / 7.3, 300^2 15.7 / 19, 512^2 25 / 25). The
 // FP64 transfer is bound by its pipe and gains earlier from warps of like lengths (64^2 62.8 / 64 ms,
@@ -1120,7 +1120,9 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
             rv = probe_steps(c, cam, ctr, rec, chunk, ar);
             if (rv) return rv;
         }
-        if (c->have_steps && nrays >= (form == RT_FP64 ? kOrderMinRaysFp64 : kOrderMinRays)) {
+        // an image in parts keeps the order at any size: dealt, no part outgrows its share of the arena
+        const bool parts = ovl || Kseq > 1;
+        if (c->have_steps && (parts || nrays >= (form == RT_FP64 ? kOrderMinRaysFp64 : kOrderMinRays))) {
             if (c->order_K != Lord.K || c->order_W != Lord.W) {
                 launch_order_build(c->d_steps, Lord, c->d_ohist, c->d_order, c->stream);
                 CK(cudaGetLastError());
