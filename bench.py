@@ -450,8 +450,9 @@ def main():
             kt_geo.append(counters["ms_geodesic"])
             kt_xf.append(counters["ms_transfer"])
             # the geodesic and transfer launches, and the two image-sum kernels
-            # (a transfer is two kernels, the points and the Stokes chain; with the staged fetch one)
-            per_xfer = 1 if args.fetch == "staged" and args.form == "mixed" else 2
+            # (a transfer is two kernels, the points and the Stokes chain, and in FP64 the one-lane kernel
+            # that returns where these have run; with the staged fetch one)
+            per_xfer = 3 if args.form == "fp64" else 1 if args.fetch == "staged" else 2
             launches += counters["geodesic_launches"] + per_xfer * counters["transfer_launches"] + 2
         e1.record(stream)
         torch.cuda.synchronize()

@@ -182,7 +182,10 @@ int rt_set_integrator(rt_ctx *ctx, double eps, int nmax);
 int rt_set_workspace(rt_ctx *ctx, void *dev_ptr, size_t bytes);
 size_t rt_workspace_min_bytes(void);
 /* Workspace size the library would use for the current camera: every ray's path at once, as
- * the streamed overlapped shape needs (a sizing hint; smaller workspaces render in chunks). */
+ * the streamed overlapped shape needs (a sizing hint; smaller workspaces render in chunks).
+ * RT_FP64 keeps records of half a path's size in what the paths leave of it, which is enough at
+ * the default step; at steps so small that it is not, the image takes two chunks. (The library's own
+ * workspace is half as large again for RT_FP64.) */
 int rt_workspace_hint(const rt_ctx *ctx, size_t *bytes);
 
 /* Render the IQUV image: out_iquv holds nx*ny*4 values, row-major [iy][ix][I,Q,U,V]

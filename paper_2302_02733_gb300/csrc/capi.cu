@@ -337,9 +337,9 @@ int rt_set_workspace(rt_ctx *c, void *dev_ptr, size_t bytes) {
 constexpr size_t kSurBlockBytes = (size_t)kBlockStates * (16 + 32 + 4);
 constexpr size_t kSurPerRayBytes = kPerRayBytes + (size_t)kBudgetBlocksPerRay * kSurBlockBytes;
 
-// Bytes per arena block the FP64 form's one-pass transfer adds: the 4 doubles of each state's record
-// that its 64 bytes do not hold (XferArgs::ext).
-constexpr size_t kExtBlockBytes = (size_t)kBlockStates * 4 * sizeof(double);
+// Bytes per arena block of the FP64 form's records: the 4 doubles of each state's that its 64 bytes do not
+// hold (record_tail).
+constexpr size_t kRecBlockBytes = (size_t)kBlockStates * 4 * sizeof(double);
 
 // Workspace bytes the streamed shape needs for nrays rays: counters, chunk counts, ray records
 // and the arena at the per-ray budget (per_ray: kPerRayBytes, or kSurPerRayBytes for the
@@ -1017,7 +1017,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
 
     // workspace carving; the surrogate form adds, per saved state, the network's inputs and
     // outputs (16 + 32 bytes)
-    size_t per_ray = kPerRayBytes + (sur ? (size_t)kBudgetBlocksPerRay * kBlockStates * 48 : 0);
+    const size_t per_ray = kPerRayBytes + (sur ? (size_t)kBudgetBlocksPerRay * kBlockStates * 48 : 0);
 
     // launch shape: the configured one, or automatic. RT_MIXED and RT_UNPOL overlap images of
     // 2^19 rays or more: streamed (chunks of about 2^15 rays, the geodesic at its own occupancy)
@@ -1038,12 +1038,6 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     // that hold a chunk each, with their own counters
     int rv = RT_OK, P = ovl ? plan_pieces(c, nrays, sur ? kSurPerRayBytes : kPerRayBytes) : 0, Kp = 0;
     const bool streamed = P > 0;
-    // the FP64 form in one pass: room for the transfer's records, unless a caller's workspace
-    // cannot hold one ray with them
-    bool ext = form == RT_FP64 && !ovl;
-    if (ext && c->ws && !c->ws_owned)
-        ext = c->ws_bytes > align_up(sizeof(Counters)) + 4 * kAlign + per_ray + kBudgetBlocksPerRay * kExtBlockBytes;
-    if (ext) per_ray += kBudgetBlocksPerRay * kExtBlockBytes;
     ChunkLayout L{nrays, 1, 1};
     if (streamed) {
         // contiguous ranges of each piece's longest-first order; the automatic shape takes finer
@@ -1057,7 +1051,8 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
         if (ovl)
             ws_rays = 2 * ChunkLayout{nrays, chunks, W}.max_size() +
                       2 * (long long)((align_up(sizeof(Counters)) + 6 * kAlign + per_ray - 1) / per_ray) + 1;
-        rv = ensure_workspace(c, ws_rays, per_ray);
+        // the FP64 form in one pass: the transfer's records too, for paths of the whole budget
+        rv = ensure_workspace(c, ws_rays, per_ray + (form == RT_FP64 && !ovl ? kBudgetBlocksPerRay * kRecBlockBytes : 0));
         if (rv) return rv;
         if (ovl) {
             // a workspace too small for kMaxChunks (256) overlapped chunks (a caller's, or a
@@ -1074,13 +1069,23 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     // the layout {n, Kseq, 1} (chunk k from k (n / Kseq) + min(k, n % Kseq)), so that with the
     // longest-first order every chunk holds the same mix of lengths and none outgrows the
     // arena's per-ray budget
-    const size_t per_block = kBlockBytes + (sur ? (size_t)kBlockStates * 48 : 0) + (ext ? kExtBlockBytes : 0);
+    const size_t per_block = kBlockBytes + (sur ? (size_t)kBlockStates * 48 : 0);
     char *base = (char *)c->ws;
     Counters *ctr = (Counters *)base;
     size_t off = align_up(sizeof(Counters));
     size_t room = c->ws_bytes - off - 3 * kAlign;
     long long chunk = std::min<long long>(nrays, (long long)(room / per_ray));
     if (chunk < 1) return RT_ERR_NOMEM;
+    // FP64 records have room in what a chunk's paths leave of their budget when they take under two
+    // thirds of it. An image in several chunks gets chunks with room for both at the whole budget, and so
+    // does one that just fits if its paths, of about (2 ln r_cam + 3.5) / eps steps, are longer than that.
+    // (Images at the hinted size in one chunk and in two: ADAF 64^2 15.1 and 27.9 ms, torus 300^2 121 and
+    // 141.) A workspace without room for one ray and its records takes the one-lane kernel.
+    const long long chunk_rec = (long long)(room / (per_ray + kBudgetBlocksPerRay * kRecBlockBytes));
+    const bool records = form == RT_FP64 && !ovl && chunk_rec > 0;
+    if (records && chunk_rec < nrays &&
+        (chunk < nrays || 3.0 * ((2.0 * std::log(cam.r_cam) + 3.5) / cam.eps / kBlockStates + 1.0) > 2.0 * kBudgetBlocksPerRay))
+        chunk = chunk_rec;
     const long long Kseq = (nrays + chunk - 1) / chunk;
 
     RayRecord *rec = (RayRecord *)(base + off);
@@ -1097,11 +1102,6 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
         feat = (float4 *)(base + off);
         off = align_up(off + (size_t)nblocks * kBlockStates * sizeof(float4));
         sur_y = (float *)(base + off);
-    }
-    double *d_ext = nullptr;
-    if (ext) {
-        off = align_up(off + (size_t)nblocks * kBlockBytes);
-        d_ext = (double *)(base + off);
     }
 
     // ray order: longest first once a render of this camera has recorded its step counts, or,
@@ -1191,7 +1191,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
             xa.pix_list = ray_list;
             xa.kt = kappa_tables(c->d_kap);
             xa.therm = c->d_therm;
-            xa.ext = d_ext;
+            xa.records = records;
             if (sur) set_surrogate_args(c, xa, feat, sur_y);
             if (k == 0) CK(cudaEventRecord(c->ev[0], c->stream));
             launch_geodesic(ga, geo_grid, c->stream);

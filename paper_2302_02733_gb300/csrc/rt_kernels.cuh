@@ -100,8 +100,7 @@ struct XferArgs {
     const JobDev *jobs;   // optional: a table of images (see GeoArgs)
     int njobs;
     const double *therm;  // FP64: the thermal tables (ThermTab)
-    double *ext;          // FP64: 4 doubles per saved state for the points' records, or NULL (then one
-                          // kernel does the whole transfer)
+    bool records;         // FP64: two kernels where the arena has room for the points' records (record_tail)
 };
 
 // ---- batched rendering: many images in one persistent launch ----------------------------

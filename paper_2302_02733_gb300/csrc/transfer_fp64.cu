@@ -2,28 +2,17 @@
 #include "transfer_kernel.cuh"
 
 namespace prt {
-template <int CM, bool JOBS>
+template <int CM>
 static void launch_two(const XferArgs &a, int grid, cudaStream_t s) {
     cudaMemsetAsync(&a.ctr->chain_next, 0, sizeof(unsigned long long), s);
     constexpr int T = PointsCfg<double>::threads;
     static_assert(T == kXferThreads, "grid counts blocks of kXferThreads");
-    points_kernel<double, CM, JOBS><<<ray_grid(grid, a.nrays, T / 32), T, 0, s>>>(a);
-    chain_kernel<double, double, JOBS><<<ray_grid(2 * grid, a.nrays, kXferThreads), kXferThreads, 0, s>>>(a);
+    points_kernel<double, CM><<<ray_grid(grid, a.nrays, T / 32), T, 0, s>>>(a);
+    chain_kernel<double, double><<<ray_grid(2 * grid, a.nrays, kXferThreads), kXferThreads, 0, s>>>(a);
 }
 void launch_transfer_fp64(const XferArgs &a, int coef, int grid, cudaStream_t s) {
-    if (a.ext) {
-        switch (coef) {
-            case 0:
-                if (a.jobs)
-                    launch_two<0, true>(a, grid, s);
-                else
-                    launch_two<0, false>(a, grid, s);
-                break;
-            case 1: launch_two<1, false>(a, grid, s); break;
-            default: break;
-        }
-        return;
-    }
+    // which of the two does the work is decided on the device; the other's kernels return at once
+    if (a.records) coef == 0 ? launch_two<0>(a, grid, s) : launch_two<1>(a, grid, s);
     grid = ray_grid(grid, a.nrays, kXferThreads);
     switch (coef) {
         case 0:

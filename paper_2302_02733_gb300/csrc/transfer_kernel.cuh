@@ -8,7 +8,7 @@
 // of screen from one emitting point to the next depend on the geometry alone. So the transfer is
 // two kernels: points_kernel, one warp per ray and one lane per saved state, 32 at a time, replaces
 // each state by its step's record (XRec); chain_kernel, one lane per ray, applies the records in
-// turn. transfer_kernel, one lane per ray for both, runs where the records have no room. Against it
+// turn. transfer_kernel, one lane per ray for both, runs where the FP64 records have no room. Against it
 // (geodesic excluded): 64^2 mixed 5.8 -> 1.4 ms, 300^2 12 -> 6.0, 1024^2 69 -> 61, and in FP64
 // 64^2 ADAF 63 -> 16 ms, 126 x 130 torus 72 -> 31, 300^2 184 -> 141.
 #pragma once
@@ -72,6 +72,14 @@ template <typename R>
 struct XRec {
     R d11, d12, d21, d22, tau, aQ, aV, rQ, rV, J0, J1, J3;
 };
+
+// FP64: the second parts of the states' records (4 doubles each) lie behind the arena blocks that the
+// chunk's rays took, in what they left of their budget; NULL where that is less than half of what they took
+// (the one-lane kernel then runs). 12 of 20 blocks are usual at the default step.
+__device__ __forceinline__ double *record_tail(const XferArgs &p) {
+    const unsigned long long used = p.ctr->arena_next;
+    return 3 * used <= 2 * (unsigned long long)p.arena.nblocks ? reinterpret_cast<double *>(p.arena.states + used * kBlockStates) : nullptr;
+}
 
 // The 2x2 matrix C_{ij} = f_i . E_j from the screen (E1, E2) to the screen (f1, f2) given as lowered
 // legs, used once, at the camera: C = (c11, c12, c21, c22).
@@ -565,6 +573,7 @@ __device__ __forceinline__ const double *thermal_weights(double *, const double 
 // outputs; otherwise over the one image of p.cam, p.model, p.out.
 template <typename R, typename OutT, int CM = 0, bool JOBS = false>
 __global__ void __launch_bounds__(kXferThreads, sizeof(R) == 4 ? 4 : 1) transfer_kernel(XferArgs p) {
+    if (sizeof(R) == 8 && p.records && record_tail(p)) return;  // the two kernels have run
     __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
     const R *sgw = thermal_weights(wsh, p.therm);
     __syncthreads();
@@ -644,9 +653,9 @@ __global__ void __launch_bounds__(kXferThreads, sizeof(R) == 4 ? 4 : 1) transfer
 
 // ---- The transfer as two kernels -------------------------------------------------------------
 // A state's record, in place of the state (64 bytes: in FP32 the 12 values, in FP64 the first 8,
-// the other 4 in p.ext), and a ray's camera matrix in place of its last state, which no step leaves.
+// the other 4 at tail), and a ray's camera matrix in place of its last state, which no step leaves.
 template <typename R>
-__device__ __forceinline__ void store_rec(const XferArgs &p, long long st, const XRec<R> &x) {
+__device__ __forceinline__ void store_rec(const XferArgs &p, double *tail, long long st, const XRec<R> &x) {
     if constexpr (sizeof(R) == 4) {
         float4 *d = reinterpret_cast<float4 *>(p.arena.states + st);
         d[0] = make_float4(x.d11, x.d12, x.d21, x.d22);
@@ -656,18 +665,18 @@ __device__ __forceinline__ void store_rec(const XferArgs &p, long long st, const
         double4_32a *d = reinterpret_cast<double4_32a *>(p.arena.states + st);
         d[0] = make_double4_32a(x.d11, x.d12, x.d21, x.d22);
         d[1] = make_double4_32a(x.tau, x.aQ, x.aV, x.rQ);
-        reinterpret_cast<double4_32a *>(p.ext)[st] = make_double4_32a(x.rV, x.J0, x.J1, x.J3);
+        reinterpret_cast<double4_32a *>(tail)[st] = make_double4_32a(x.rV, x.J0, x.J1, x.J3);
     }
 }
 template <typename R>
-__device__ __forceinline__ XRec<R> load_rec(const XferArgs &p, long long st) {
+__device__ __forceinline__ XRec<R> load_rec(const XferArgs &p, const double *tail, long long st) {
     if constexpr (sizeof(R) == 4) {
         const float4 *d = reinterpret_cast<const float4 *>(p.arena.states + st);
         const float4 a = d[0], b = d[1], c = d[2];
         return XRec<R>{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
     } else {
         const double4_32a *d = reinterpret_cast<const double4_32a *>(p.arena.states + st);
-        const double4_32a a = d[0], b = d[1], c = reinterpret_cast<const double4_32a *>(p.ext)[st];
+        const double4_32a a = d[0], b = d[1], c = reinterpret_cast<const double4_32a *>(tail)[st];
         return XRec<R>{a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
     }
 }
@@ -725,6 +734,8 @@ struct PointsCfg<double> {
 // handed down lane by lane.
 template <typename R, int CM = 0, bool JOBS = false>
 __global__ void __launch_bounds__(PointsCfg<R>::threads, PointsCfg<R>::blocks) points_kernel(XferArgs p) {
+    double *const tail = sizeof(R) == 8 ? record_tail(p) : nullptr;
+    if (sizeof(R) == 8 && !tail) return;
     __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
     const R *sgw = thermal_weights(wsh, p.therm);
     __syncthreads();
@@ -806,7 +817,7 @@ __global__ void __launch_bounds__(PointsCfg<R>::threads, PointsCfg<R>::blocks) p
                 xfer_link(P, T0, in, x);
             else
                 x.tau = R(-INFINITY);
-            store_rec(p, st, x);
+            store_rec(p, tail, st, x);
         }
         if (base == 0 && lane == 0) {
             int ix, iy;
@@ -834,6 +845,8 @@ __global__ void __launch_bounds__(PointsCfg<R>::threads, PointsCfg<R>::blocks) p
 // over the records of points_kernel; the next record is loaded before the current one is applied.
 template <typename R, typename OutT, bool JOBS = false>
 __global__ void __launch_bounds__(kXferThreads) chain_kernel(XferArgs p) {
+    const double *const tail = sizeof(R) == 8 ? record_tail(p) : nullptr;
+    if (sizeof(R) == 8 && !tail) return;
     long long ray = -1;
     int blk = -1, slot = 0, n = 0, rstat = 0, job = 0;
     bool live = false, drained = false;
@@ -854,7 +867,7 @@ __global__ void __launch_bounds__(kXferThreads) chain_kernel(XferArgs p) {
             blk = p.arena.prev[blk];
             slot = kBlockStates - 1;
         }
-        next = load_rec<R>(p, (long long)blk * kBlockStates + slot);
+        next = load_rec<R>(p, tail, (long long)blk * kBlockStates + slot);
     };
     for (;;) {
         bool want = !live && !drained;
