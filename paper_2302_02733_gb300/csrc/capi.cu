@@ -125,7 +125,6 @@ int rt_create(rt_ctx **out, int device, void *stream) {
     c->staged_bps = transfer_blocks_per_sm_staged();
     c->pipe_bps[0] = pipe_blocks_per_sm_fp64();
     c->pipe_bps[1] = pipe_blocks_per_sm_mixed();
-    c->geo_regs = geodesic_regs();
     c->xf_regs_fp64 = transfer_regs_fp64();
     c->xf_regs_mixed = transfer_regs_mixed();
     c->regs_per_sm = prop.regsPerMultiprocessor;
@@ -519,7 +518,7 @@ static int probe_steps(rt_ctx *c, const Camera &cam, Counters *ctr, RayRecord *r
     GeoArgs ga{cam, c->d_sctab, ar, rec, ctr, np, 0};
     ga.pix_list = c->d_probe;
     ga.steps_out = c->d_steps;
-    launch_geodesic(ga, c->nsm * c->geo_bps, c->stream);
+    launch_geodesic(ga, c->nsm, c->geo_bps, c->stream);
     launch_steps_fill(c->d_steps, cam.nx, cam.ny, kProbeStride, c->stream);
     CK(cudaGetLastError());
     c->have_steps = true;
@@ -547,11 +546,11 @@ static ChunkLayout overlap_chunks(const rt_ctx *c, long long nrays, int chunks, 
 }
 
 // Registers of a block (allocated per warp, in units of 256) and the transfer blocks per SM that
-// fit in the register file beside geo_b geodesic blocks, at most xf_b (0: none).
+// fit in the register file beside geo_b geodesic blocks of a launch of nrays, at most xf_b (0: none).
 static int block_regs(int regs, int threads) { return ((regs * 32 + 255) / 256) * 256 * ((threads + 31) / 32); }
-static int xf_beside_geo(const rt_ctx *c, int form, int geo_b, int xf_b) {
+static int xf_beside_geo(const rt_ctx *c, int form, long long nrays, int geo_b, int xf_b) {
     const int xr = block_regs(form == RT_FP64 ? c->xf_regs_fp64 : c->xf_regs_mixed, kXferThreads);
-    const int room = c->regs_per_sm - geo_b * block_regs(c->geo_regs, kGeoThreads);
+    const int room = c->regs_per_sm - geo_b * block_regs(geodesic_regs(nrays, c->nsm), kGeoThreads);
     const int fit = room > 0 ? room / xr : 0;
     return std::min(xf_b, fit);
 }
@@ -565,7 +564,7 @@ static int xf_beside_geo(const rt_ctx *c, int form, int geo_b, int xf_b) {
 // RT_ERR_NOMEM when a half cannot hold a chunk of at most kMaxChunks-th of the rays.
 static int render_overlap(rt_ctx *c, int form, int coef, const Camera &cam, const Model &mod, const int *list,
                           uint16_t *steps_out, const ChunkLayout &L, void *d_out, uint8_t *d_status,
-                          void *d_depth, int geo_grid, int xf_grid, const JobDev *jobs = nullptr, int njobs = 0) {
+                          void *d_depth, int geo_b, int xf_grid, const JobDev *jobs = nullptr, int njobs = 0) {
     const long long K = L.K;
     const bool sur = form == RT_SURROGATE;
     // per arena block: the states and the prev link, and for the surrogate form the network's
@@ -624,7 +623,7 @@ static int render_overlap(rt_ctx *c, int form, int coef, const Camera &cam, cons
         xa.njobs = njobs;
         if (sur) set_surrogate_args(c, xa, feat[h], sur_y[h]);
         CK(cudaEventRecord(gs[i], sg));
-        launch_geodesic(ga, geo_grid, sg);
+        launch_geodesic(ga, c->nsm, geo_b, sg);
         CK(cudaEventRecord(ge[i], sg));
         CK(cudaStreamWaitEvent(st, ge[i], 0));
         CK(cudaEventRecord(ts[i], st));
@@ -721,7 +720,7 @@ constexpr double kStreamWaitSeconds = 600.0;
 // a transfer is launched after the host has seen its chunks' flags.
 static int render_streamed(rt_ctx *c, int form, int coef, const Camera &cam, const Model &mod, const int *list,
                            uint16_t *steps_out, long long nrays, int P, int K, void *d_out, uint8_t *d_status,
-                           void *d_depth, int geo_grid, int xf_grid, int xf_grid_alone, const JobDev *jobs = nullptr,
+                           void *d_depth, int geo_b, int xf_grid, int xf_grid_alone, const JobDev *jobs = nullptr,
                            int njobs = 0) {
     int rv = ensure_overlap(c);
     if (rv) return rv;
@@ -793,7 +792,7 @@ static int render_streamed(rt_ctx *c, int form, int coef, const Camera &cam, con
         ga.chunk_flag = c->d_flags;
         ga.layout = L;
         CK(cudaEventRecord(gs[p], sg));
-        if (n_p > 0) launch_geodesic(ga, geo_grid, sg);
+        if (n_p > 0) launch_geodesic(ga, c->nsm, geo_b, sg);
         CK(cudaEventRecord(ge[p], sg));
         CK(cudaGetLastError());
 
@@ -929,7 +928,8 @@ int render_jobs_overlap(rt_ctx *c, int form, const JobDev *d_jobs, const JobDev 
     const long long K = L.K;
     int rv = RT_OK;
     const int xf_own = form == RT_FP64 ? c->fp64_bps : c->mixed_bps, geo_b = streamed ? c->geo_bps : 1;
-    const int geo_grid = c->nsm * geo_b, xf_grid = c->nsm * std::max(streamed ? 0 : 1, xf_beside_geo(c, form, geo_b, xf_own));
+    const long long geo_rays = streamed ? ChunkLayout{nrays, P, 1}.max_size() : L.max_size();
+    const int xf_grid = c->nsm * std::max(streamed ? 0 : 1, xf_beside_geo(c, form, geo_rays, geo_b, xf_own));
     // longest first, as for one image, once a batch of the same cameras has recorded its steps
     unsigned long long key = 1469598103934665603ull;  // FNV-1a over the cameras and integrator
     auto mix = [&](const void *v, size_t n) {
@@ -978,10 +978,10 @@ int render_jobs_overlap(rt_ctx *c, int form, const JobDev *d_jobs, const JobDev 
     }
     if (streamed)
         rv = render_streamed(c, form, 0, h_jobs[0].cam, h_jobs[0].model, list, c->d_bsteps, nrays, P, Kp, nullptr,
-                             nullptr, nullptr, geo_grid, xf_grid, c->nsm * xf_own, d_jobs, njobs);
+                             nullptr, nullptr, geo_b, xf_grid, c->nsm * xf_own, d_jobs, njobs);
     else
         rv = render_overlap(c, form, 0, h_jobs[0].cam, h_jobs[0].model, list, c->d_bsteps, L, nullptr, nullptr,
-                            nullptr, geo_grid, xf_grid, d_jobs, njobs);
+                            nullptr, geo_b, xf_grid, d_jobs, njobs);
     if (rv) return rv;
     c->last_rays = nrays;
     c->last_was_overlap = true;
@@ -1159,19 +1159,19 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
 
     const int xf_max = form == RT_FP64 ? c->fp64_bps : c->mixed_bps;
     const int geo_bps = geo_b > 0 ? geo_b : c->geo_bps;
-    const int geo_grid = c->nsm * geo_bps;
     const int xf_own = c->rcfg.xfer_blocks_per_sm > 0 ? std::min(c->rcfg.xfer_blocks_per_sm, xf_max) : xf_max;
     // overlapped: no more transfer blocks per SM than fit beside the geodesic's (streamed: none
     // before the geodesic has ended, where none fit)
-    const int xf_grid = c->nsm * (ovl ? std::max(streamed ? 0 : 1, xf_beside_geo(c, form, geo_bps, xf_own)) : xf_own);
+    const long long geo_rays = streamed ? ChunkLayout{nrays, P, 1}.max_size() : L.max_size();
+    const int xf_grid = c->nsm * (ovl ? std::max(streamed ? 0 : 1, xf_beside_geo(c, form, geo_rays, geo_bps, xf_own)) : xf_own);
     c->last_was_overlap = false;
     c->last_was_streamed = false;
     if (ovl) {
         if (streamed)
             rv = render_streamed(c, form, coef, cam, mod, ray_list, steps_out, nrays, P, Kp, d_out, d_status, d_depth,
-                                 geo_grid, xf_grid, c->nsm * xf_own);
+                                 geo_bps, xf_grid, c->nsm * xf_own);
         else
-            rv = render_overlap(c, form, coef, cam, mod, ray_list, steps_out, L, d_out, d_status, d_depth, geo_grid,
+            rv = render_overlap(c, form, coef, cam, mod, ray_list, steps_out, L, d_out, d_status, d_depth, geo_bps,
                                 xf_grid);
         if (rv) return rv;
         c->last_was_overlap = true;
@@ -1194,7 +1194,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
             xa.records = records;
             if (sur) set_surrogate_args(c, xa, feat, sur_y);
             if (k == 0) CK(cudaEventRecord(c->ev[0], c->stream));
-            launch_geodesic(ga, geo_grid, c->stream);
+            launch_geodesic(ga, c->nsm, geo_bps, c->stream);
             if (sur) launch_network_pass(c, xa, sur_y, nblocks, &ctr->arena_next, xf_grid, c->stream);
             if (k == 0) CK(cudaEventRecord(c->ev[1], c->stream));
             if (form == RT_FP64)
@@ -1273,7 +1273,7 @@ int rt_render_features(rt_ctx *c, float *feat, long long cap, long long *count) 
         }
         xa.feat_raw = reinterpret_cast<float4 *>(feat);
         xa.feat_cap = cap;
-        launch_geodesic(ga, c->nsm * c->geo_bps, c->stream);
+        launch_geodesic(ga, c->nsm, c->geo_bps, c->stream);
         launch_sur_features(xa, c->nsm * c->mixed_bps, c->stream);
         CK(cudaGetLastError());
     }

@@ -193,12 +193,13 @@ int launch_geo_tables(double *tab, cudaStream_t s) {
                : -1;
 }
 
-// The rays of 2 blocks on each of the 152 SMs: up to there every ray is resident in either variant.
-constexpr long long kGeoFewRays = 2 * 152 * kGeoThreads;
+// The rays of 2 blocks on each SM: up to there every ray is resident in either variant (2 blocks of the
+// larger one always fit: that is what it is compiled for).
+static bool few_rays(long long nrays, int nsm) { return nrays <= 2ll * nsm * kGeoThreads; }
 
-void launch_geodesic(const GeoArgs &a, int grid, cudaStream_t s) {
-    grid = ray_grid(grid, a.nrays, kGeoThreads);
-    if (a.nrays <= kGeoFewRays) {
+void launch_geodesic(const GeoArgs &a, int nsm, int blocks_per_sm, cudaStream_t s) {
+    const int grid = ray_grid(nsm * blocks_per_sm, a.nrays, kGeoThreads);
+    if (few_rays(a.nrays, nsm)) {
         if (a.jobs)
             geodesic_kernel<true, 2><<<grid, kGeoThreads, 0, s>>>(a);
         else
@@ -219,8 +220,10 @@ static int func_regs(const void *f) {
     return a.numRegs;
 }
 
-int geodesic_regs() {
-    return std::max(func_regs((const void *)geodesic_kernel<false, 3>), func_regs((const void *)geodesic_kernel<true, 3>));
+int geodesic_regs(long long nrays, int nsm) {
+    return few_rays(nrays, nsm)
+               ? std::max(func_regs((const void *)geodesic_kernel<false, 2>), func_regs((const void *)geodesic_kernel<true, 2>))
+               : std::max(func_regs((const void *)geodesic_kernel<false, 3>), func_regs((const void *)geodesic_kernel<true, 3>));
 }
 
 int geodesic_blocks_per_sm() {

@@ -88,7 +88,7 @@ int rt_render_static(rt_ctx *c, int form, void *out_iquv, uint8_t *status) {
     const int geo_b = c->rcfg.geo_blocks_per_sm > 0 ? c->rcfg.geo_blocks_per_sm : c->geo_bps;
     const int xf_max = form == RT_FP64 ? c->fp64_bps : c->mixed_bps;
     const int xf_b = c->rcfg.xfer_blocks_per_sm > 0 ? std::min(c->rcfg.xfer_blocks_per_sm, xf_max) : xf_max;
-    launch_geodesic(ga, c->nsm * geo_b, c->stream);
+    launch_geodesic(ga, c->nsm, geo_b, c->stream);
     cudaEventRecord(c->ev[1], c->stream);
     xa.kt = kappa_tables(c->d_kap);
     xa.therm = c->d_therm;

@@ -50,8 +50,8 @@ struct rt_ctx {
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     long long last_rays = 0, last_blocks_total = 0;
     int geo_bps = 1, fp64_bps = 1, mixed_bps = 1;
-    // registers per thread of the geodesic and transfer kernels, and per SM
-    int geo_regs = 255, xf_regs_fp64 = 255, xf_regs_mixed = 255, regs_per_sm = 65536;
+    // registers per thread of the transfer kernels, and per SM
+    int xf_regs_fp64 = 255, xf_regs_mixed = 255, regs_per_sm = 65536;
     float last_ms_total = 0.f;
     bool last_was_batch = false;
 

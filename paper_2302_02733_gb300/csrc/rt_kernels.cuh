@@ -194,7 +194,7 @@ inline int ray_grid(int grid, long long n, int threads) {
     const long long need = n > 0 ? (n + threads - 1) / threads : 1;
     return need < grid ? (int)need : grid;
 }
-void launch_geodesic(const GeoArgs &a, int grid, cudaStream_t s);
+void launch_geodesic(const GeoArgs &a, int nsm, int blocks_per_sm, cudaStream_t s);
 // Longest-first ray order from the step counts of a previous render of the same camera:
 // order[i] is the pixel of ray i, by step count descending (16-step buckets), placed by the
 // layout L into its chunks. hist: kOrderBuckets unsigned of scratch.
@@ -230,9 +230,10 @@ int geodesic_blocks_per_sm();
 int transfer_blocks_per_sm_fp64();
 int transfer_blocks_per_sm_mixed();
 int transfer_blocks_per_sm_staged();
-// registers per thread of a kernel (cudaFuncGetAttributes), for the overlapped shape's sharing
-// of an SM's register file between one geodesic block and the transfer blocks beside it
-int geodesic_regs();
+// registers per thread of a kernel (cudaFuncGetAttributes; geodesic: of the variant that a launch of nrays
+// takes), for the overlapped shape's sharing of an SM's register file between one geodesic block and the
+// transfer blocks beside it
+int geodesic_regs(long long nrays, int nsm);
 int transfer_regs_fp64();
 int transfer_regs_mixed();  // the largest of the mixed, staged and unpolarized transfers
 
