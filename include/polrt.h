@@ -408,7 +408,9 @@ typedef struct {
 /* Launch shape of the batched form. mode 0 (RT_BATCH_PERSISTENT) is one persistent launch,
  * captured in a CUDA graph: each block has 8 warps, geo_warps of them integrate geodesics and
  * the rest run the transfer (odd-numbered blocks take geo_warps_odd instead when it is not 0,
- * so that the two roles can be balanced in steps of half a warp per block); step_tile is the number of RK4 steps a lane takes between its
+ * so that the two roles can be balanced in steps of half a warp per block). RT_MIXED gives the roles
+ * to pairs of SMs instead, in the same proportion: geo_warps + geo_warps_odd (geo_warps twice when
+ * that is 0) of every 16 pairs integrate until no ray is left. step_tile is the number of RK4 steps a lane takes between its
  * queue and pool checks; blocks_per_sm is the number of resident blocks per SM (the grid is
  * that times the SM count). mode 1 (RT_BATCH_CHUNKS) treats the rays of all images as one ray
  * space and runs it like one large image in the automatic overlapped shape of

@@ -1,13 +1,19 @@
 // The batched form: geodesics and transfers of many images in one persistent launch.
 //
-// Each 8-warp block holds both roles of the method (the paper's Section 2.1). Its first
-// geo_warps warps integrate backward geodesics and save the states. The remaining warps walk
-// completed paths toward the camera and do the transfer (FP64 or FP32). The roles share the SM: in
-// the FP64 form the FP64 pipe's transfer and the integer pipes' geodesic, in the mixed form two
-// roles on the same pipes. Six mixed images of 128^2 to 512^2 take 294 ms here at their best shape,
-// 196 with an FP64 geodesic, and 86 as one ray space in two kernels (mode 1, which the autotuner
-// takes); whole blocks of one role (275), the step as a call (283) and transfer warps that sleep
-// until most of their lanes have a ray (294) were no remedy.
+// Some warps integrate backward geodesics and save the states, the others walk completed paths toward
+// the camera and do the transfer, FP64 or FP32 (the paper's Section 2.1).
+//
+// In the FP64 form each 8-warp block holds both roles, geo_warps of them the first: the transfer
+// lives on the FP64 pipe, the geodesic on the integer pipes, and they share the SM.
+//
+// In the mixed form both live on the same pipes, and their loops together do not fit in the instruction
+// cache: a step took 85,000 clocks where the geodesic alone takes 13,900. There the roles go to pairs
+// of SMs (which share that cache), geo_warps of every 8 pairs the geodesic, handed out in the order in
+// which the pairs' first blocks start, the first two one each. Geodesic warps that find no more rays
+// transfer what is left, and one warp of their blocks is kept for the transfer should the pool run
+// dry, so that the launch needs no other SM to end. Six mixed images of 128^2 to 512^2 take 171 ms at
+// their best shape (297 with both roles in each block, 230 with a role to each SM; 197 when the geodesic
+// was FP64), and 86 as one ray space in two kernels (mode 1).
 //
 // Flow control, all in global memory:
 //  - rays come from a queue (geo_next) over all images of the batch;
@@ -305,12 +311,54 @@ __device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *sgw) {
     if (n_spin) atomicAdd(&p.ctr->free_spins, n_spin);
 }
 
+// Mixed form: whether this SM's pair integrates geodesics (one thread of the block asks).
+__device__ __forceinline__ bool pair_integrates(const PipeArgs &p) {
+    unsigned sm;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+    unsigned *slot = p.ctr->role + (sm >> 1) % kRolePairs;
+    unsigned v = atomicCAS(slot, 0u, 1u);
+    if (v == 0u) {  // of 16 pairs in turn: the first, and g of the 14 after the second
+        const unsigned k = atomicAdd(&p.ctr->role_next, 1u) & 15u, g = (unsigned)(p.geo_warps + p.geo_warps_odd) - 1u;
+        v = k == 0u || (k > 1u && (k - 1u) * g / 14u != (k - 2u) * g / 14u) ? 2u : 3u;
+        atomicExch(slot, v);
+    }
+    // the block that chooses is between two instructions; a wait that runs out leaves the transfer
+    for (int spin = 0; v == 1u && spin < kRingSpin; spin++) v = atomicAdd(slot, 0u);
+    return v == 2u;
+}
+
+// Mixed form, the last warp of a geodesic block: asleep until every ray is taken, or a lane waits for a path
+// block (more tickets than returns), or for kReadyWaitNs.
+__device__ __forceinline__ void pipe_reserve(const PipeArgs &p) {
+    const unsigned long long t0 = global_ns();
+    volatile unsigned long long *next = &p.ctr->geo_next, *head = &p.ctr->pool_head, *tail = &p.ctr->pool_tail;
+    for (;;) {
+        int go = 0;
+        if ((threadIdx.x & 31) == 0) go = *next >= (unsigned long long)p.nrays || *head > *tail || global_ns() - t0 > kReadyWaitNs;
+        if (__shfl_sync(0xffffffffu, go, 0)) break;
+        __nanosleep(20000);
+    }
+}
+
 template <typename R, typename OutT>
 __global__ void __launch_bounds__(kPipeThreads, sizeof(R) == 4 ? 2 : 1) pipe_kernel(PipeArgs p) {
     __shared__ R wsh[sizeof(R) == 4 ? 32 : 1];
     __shared__ __align__(16) fx64 fxtab[2 * kFxTab];  // the geodesic's sin/cos table
     const R *sgw = thermal_weights(wsh, p.therm);
     load_fx_table(p.sctab, fxtab);
+    if constexpr (sizeof(R) == 4) {
+        __shared__ bool integrates;
+        if (threadIdx.x == 0) integrates = pair_integrates(p);
+        __syncthreads();
+        if (integrates) {
+            if ((threadIdx.x >> 5) < kPipeThreads / 32 - 1)
+                pipe_geodesic(p, GeoTabs{fxtab, p.sctab});
+            else
+                pipe_reserve(p);
+        }
+        pipe_transfer<R, OutT>(p, sgw);
+        return;
+    }
     __syncthreads();
     if ((int)(threadIdx.x >> 5) < ((blockIdx.x & 1) ? p.geo_warps_odd : p.geo_warps))
         pipe_geodesic(p, GeoTabs{fxtab, p.sctab});

@@ -137,6 +137,7 @@ struct Pool {
     int nblocks;
 };
 
+constexpr int kRolePairs = 128;
 struct PipeCounters {
     unsigned long long geo_next, xfer_next, ready_tail;  // work queues
     unsigned long long pool_head, pool_tail;             // free-ring ticket and return positions
@@ -150,6 +151,9 @@ struct PipeCounters {
     // and polls of a busy slot when returning a block
     unsigned long long geo_iters, geo_sleeps, xfer_iters, xfer_sleeps;
     unsigned long long ticket_polls, ready_polls, free_spins, tickets;
+    // mixed form: roles handed out so far, and each SM pair's: 0 none yet, 1 being chosen, 2 geodesic,
+    // 3 transfer
+    unsigned int role_next, role[kRolePairs];
 };
 constexpr unsigned kPipeErrRing = 1u;   // a free-ring slot never changed
 constexpr unsigned kPipeErrReady = 2u;  // a transfer lane never received its ray
