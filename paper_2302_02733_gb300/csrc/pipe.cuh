@@ -10,10 +10,11 @@
 // cache: a step took 85,000 clocks where the geodesic alone takes 13,900. There the roles go to pairs
 // of SMs (which share that cache), geo_warps of every 8 pairs the geodesic, handed out in the order in
 // which the pairs' first blocks start, the first two one each. Geodesic warps that find no more rays
-// transfer what is left, and one warp of their blocks is kept for the transfer should the pool run
-// dry, so that the launch needs no other SM to end. Six mixed images of 128^2 to 512^2 take 171 ms at
-// their best shape (297 with both roles in each block, 230 with a role to each SM; 197 when the geodesic
-// was FP64), and 86 as one ray space in two kernels (mode 1).
+// transfer what is left, and one warp of each such pair is kept for the transfer should the pool run
+// dry, so that the launch needs no other SM to end. Six mixed images of 128^2 to 512^2 take 163 ms at
+// their best shape, 96 images 2.9 s (297 ms and 5.4 s with both roles in each block, 230 ms with a role to
+// each SM, 167 ms and 3.7 s with a warp kept in every block; 197 ms and 3.4 s when the geodesic was
+// FP64), and 86 ms and 1.5 s as one ray space in two kernels (mode 1).
 //
 // Flow control, all in global memory:
 //  - rays come from a queue (geo_next) over all images of the batch;
@@ -311,12 +312,14 @@ __device__ __forceinline__ void pipe_transfer(const PipeArgs &p, const R *sgw) {
     if (n_spin) atomicAdd(&p.ctr->free_spins, n_spin);
 }
 
-// Mixed form: whether this SM's pair integrates geodesics (one thread of the block asks).
-__device__ __forceinline__ bool pair_integrates(const PipeArgs &p) {
+// Mixed form: how many of this block's warps integrate geodesics: none where its SM's pair transfers, else
+// all, but one in the block that the pair's role was chosen for (one thread of the block asks).
+__device__ __forceinline__ int pair_role(const PipeArgs &p) {
     unsigned sm;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
     unsigned *slot = p.ctr->role + (sm >> 1) % kRolePairs;
     unsigned v = atomicCAS(slot, 0u, 1u);
+    const int geo = kPipeThreads / 32 - (v == 0u);
     if (v == 0u) {  // of 16 pairs in turn: the first, and g of the 14 after the second
         const unsigned k = atomicAdd(&p.ctr->role_next, 1u) & 15u, g = (unsigned)(p.geo_warps + p.geo_warps_odd) - 1u;
         v = k == 0u || (k > 1u && (k - 1u) * g / 14u != (k - 2u) * g / 14u) ? 2u : 3u;
@@ -324,10 +327,10 @@ __device__ __forceinline__ bool pair_integrates(const PipeArgs &p) {
     }
     // the block that chooses is between two instructions; a wait that runs out leaves the transfer
     for (int spin = 0; v == 1u && spin < kRingSpin; spin++) v = atomicAdd(slot, 0u);
-    return v == 2u;
+    return v == 2u ? geo : 0;
 }
 
-// Mixed form, the last warp of a geodesic block: asleep until every ray is taken, or a lane waits for a path
+// Mixed form, the warp left over in a geodesic pair: asleep until every ray is taken, or a lane waits for a path
 // block (more tickets than returns), or for kReadyWaitNs.
 __device__ __forceinline__ void pipe_reserve(const PipeArgs &p) {
     const unsigned long long t0 = global_ns();
@@ -347,15 +350,13 @@ __global__ void __launch_bounds__(kPipeThreads, sizeof(R) == 4 ? 2 : 1) pipe_ker
     const R *sgw = thermal_weights(wsh, p.therm);
     load_fx_table(p.sctab, fxtab);
     if constexpr (sizeof(R) == 4) {
-        __shared__ bool integrates;
-        if (threadIdx.x == 0) integrates = pair_integrates(p);
+        __shared__ int geo;
+        if (threadIdx.x == 0) geo = pair_role(p);
         __syncthreads();
-        if (integrates) {
-            if ((threadIdx.x >> 5) < kPipeThreads / 32 - 1)
-                pipe_geodesic(p, GeoTabs{fxtab, p.sctab});
-            else
-                pipe_reserve(p);
-        }
+        if ((int)(threadIdx.x >> 5) < geo)
+            pipe_geodesic(p, GeoTabs{fxtab, p.sctab});
+        else if (geo > 0)
+            pipe_reserve(p);
         pipe_transfer<R, OutT>(p, sgw);
         return;
     }
