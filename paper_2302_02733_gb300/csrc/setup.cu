@@ -30,7 +30,7 @@ void launch_x2_table(const GridModel &g, double *table, float *table_f, cudaStre
 }
 
 // The FP64 tables of ThermTab: on each segment the functions at the D + 1 Chebyshev nodes (one thread
-// each), then the coefficients in u (one thread a function).
+// each), their Chebyshev coefficients (one a thread), and from those the powers of u (one thread a function).
 __device__ void bessel_ratio_values(double Te, double v[2]) {
     // K_n(z) e^z = int_0^inf e^{-2 z sinh^2(t/2)} cosh(n t) dt by the trapezoid rule
     const double z = 1.0 / Te, h = 0.125 * fmin(1.0, rsqrt(z));
@@ -54,14 +54,19 @@ __device__ void shcherbakov_values(double X, double v[2]) {
 constexpr int kThermPerBlock = 16;
 template <int D, void (*fn)(double, double *)>
 __global__ void therm_table_kernel(double *tab, int bits, int e0) {
-    __shared__ double f[2][kThermPerBlock][D + 1];
+    __shared__ double f[2][kThermPerBlock][D + 1], ch[2][kThermPerBlock][D + 1];
     const int li = threadIdx.x / (D + 1), j = threadIdx.x % (D + 1), i = blockIdx.x * kThermPerBlock + li;
     double v[2];
     fn(ThermTab::at(i, bits, e0, cospi((j + 0.5) / (D + 1))), v);
     f[0][li][j] = v[0];
     f[1][li][j] = v[1];
     __syncthreads();
-    if (j < 2) therm_fit<D>(f[j][li], tab + (2 * i + j) * (D + 1));
+    for (int m = 0; m < 2; m++) ch[m][li][j] = therm_chebyshev<D>(f[m][li], j);
+    __syncthreads();
+    if (j >= 2) return;
+    double p[D + 1];
+    therm_powers<D>(ch[j][li], p);
+    for (int q = 0; q <= D; q++) tab[(2 * i + j) * (D + 1) + q] = p[q];
 }
 
 int launch_thermal_tables(double *buf, cudaStream_t s) {

@@ -52,17 +52,22 @@ struct ThermTab {
     }
 };
 
-// Coefficients in u of the polynomial through f at the Chebyshev nodes x_j = cos(pi (j + 1/2) / (D + 1)).
+// Chebyshev coefficient k of the polynomial through f at the nodes x_j = cos(pi (j + 1/2) / (D + 1)), and from
+// all of them the coefficients in u.
 template <int D>
-__device__ __forceinline__ void therm_fit(const double f[D + 1], double p[D + 1]) {
+__device__ __forceinline__ double therm_chebyshev(const double f[D + 1], int k) {
+    double s = 0.0;
+    for (int q = 0; q <= D; q++) s += f[q] * cospi(k * (q + 0.5) / (D + 1));
+    return s * (k == 0 ? 1.0 : 2.0) / (D + 1);
+}
+template <int D>
+__device__ __forceinline__ void therm_powers(const double ch[D + 1], double p[D + 1]) {
     double a[D + 1], b[D + 1];  // T_k and T_k+1 in powers of x = 2 u
     for (int q = 0; q <= D; q++) p[q] = 0.0, a[q] = q == 0, b[q] = q == 1;
     for (int k = 0; k <= D; k++) {
-        double s = 0.0, c[D + 1];
-        for (int q = 0; q <= D; q++) s += f[q] * cospi(k * (q + 0.5) / (D + 1));
-        s *= (k == 0 ? 1.0 : 2.0) / (D + 1);
+        double c[D + 1];
         for (int q = 0; q <= D; q++) {
-            p[q] += s * a[q];
+            p[q] += ch[k] * a[q];
             c[q] = (q > 0 ? 2.0 * b[q - 1] : 0.0) - a[q];
         }
         for (int q = 0; q <= D; q++) a[q] = b[q], b[q] = c[q];

@@ -50,13 +50,16 @@ static void shcherbakov(L X, L v[2], L sc[2]) {
 template <int D>
 static void fill(double *tab, int n, int bits, int e0, void (*fn)(L, L *, L *)) {
     for (int i = 0; i < n; i++) {
-        double f[2][D + 1];
+        double f[2][D + 1], ch[D + 1];
         for (int j = 0; j <= D; j++) {
             L v[2], s[2];
             fn(T::at(i, bits, e0, cospi((j + 0.5) / (D + 1))), v, s);
             f[0][j] = (double)v[0], f[1][j] = (double)v[1];
         }
-        for (int m = 0; m < 2; m++) therm_fit<D>(f[m], tab + (2 * i + m) * (D + 1));
+        for (int m = 0; m < 2; m++) {
+            for (int k = 0; k <= D; k++) ch[k] = therm_chebyshev<D>(f[m], k);
+            therm_powers<D>(ch, tab + (2 * i + m) * (D + 1));
+        }
     }
 }
 int main() {
