@@ -338,7 +338,7 @@ int rt_image_visibilities(rt_ctx *ctx, const void *img, int form, int stokes, vo
  * one pass of each kernel. RT_SURROGATE overlaps when chunks >= 2 is set: streamed, each
  * transfer launch's rays go through the features pass, the network (over compact rows) and
  * the transfer in turn; in halves, per chunk (both measured slower than one pass on GB300).
- * Independently of the shape, a full render of 2^17 rays or more records each
+ * Independently of the shape, a full render of 2^17 rays or more (RT_FP64: 2^13) records each
  * pixel's step count, and the next render of the same camera and integrator takes its rays
  * longest first, so that no launch ends waiting for a few long photon-ring rays (smaller images
  * are all in flight at once and run in pixel order, unless they are rendered in parts: overlapped,

@@ -27,12 +27,12 @@ constexpr int kAutoLastDiv = 1;
 // automatic streamed shape: about 2^kStreamChunkShift rays per chunk, at least 16 per piece, the
 // geodesic at its own occupancy
 constexpr int kStreamChunkShift = 15;
-// Images of fewer rays in one part run in pixel order: they fill the lanes at most about twice, and a
-// warp of only long rays takes longer a step than one whose lanes are leaving. Whole images, pixel order
-// against longest first: mixed ADAF 128^2 6.7 / 7.4 ms, 300^2 15.4 / 16.3, 362^2 19.5 / 17.8, 512^2 32.3 /
-// 27.9, torus 300^2 21.2 / 24.7, 362^2 24.8 / 23.7, 512^2 42.1 / 38.5; FP64 ADAF 64^2 15.1 / 15.5, 181^2
-// 40.7 / 42.5, 256^2 59.5 / 63.5, 340^2 101 / 97, torus 126 x 130 31.1 / 32.9, 256^2 84 / 92, 340^2 152 / 151.
-constexpr long long kOrderMinRays = 1ll << 17;
+// Images of fewer rays in one part run in pixel order: they fill the lanes at most about twice, and a warp of
+// only long rays takes longer a step than one whose lanes are leaving (geodesics, pixel order
+// against longest first: 64^2 5.4 / 6.3 ms, 128^2 6.4 / 7.3, 300^2 15.7 / 19, 512^2 25 / 25). The
+// FP64 transfer is bound by its pipe and gains earlier from warps of like lengths (64^2 62.8 / 64 ms,
+// 126 x 130 80 / 72, 300^2 230 / 185).
+constexpr long long kOrderMinRays = 1ll << 17, kOrderMinRaysFp64 = 1ll << 13;
 // RT_FETCH_AUTO: the grid fetch measured faster on GB300 for the benchmark image
 constexpr bool kStagedByDefault = false;
 
@@ -1122,7 +1122,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
         }
         // an image in parts keeps the order at any size: dealt, no part outgrows its share of the arena
         const bool parts = ovl || Kseq > 1;
-        if (c->have_steps && (parts || nrays >= kOrderMinRays)) {
+        if (c->have_steps && (parts || nrays >= (form == RT_FP64 ? kOrderMinRaysFp64 : kOrderMinRays))) {
             if (c->order_K != Lord.K || c->order_W != Lord.W) {
                 launch_order_build(c->d_steps, Lord, c->d_ohist, c->d_order, c->stream);
                 CK(cudaGetLastError());
