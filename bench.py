@@ -451,8 +451,8 @@ def main():
             kt_xf.append(counters["ms_transfer"])
             # the geodesic and transfer launches, and the two image-sum kernels
             # (a transfer is two kernels, the points and the Stokes chain, and in FP64 the one-lane kernel
-            # that returns where these have run; with the staged fetch one)
-            per_xfer = 3 if args.form == "fp64" else 1 if args.fetch == "staged" else 2
+            # that returns where these have run; with the staged fetch, and overlapped FP64, one)
+            per_xfer = (3 if counters["shape"] == 0 else 1) if args.form == "fp64" else 1 if args.fetch == "staged" else 2
             launches += counters["geodesic_launches"] + per_xfer * counters["transfer_launches"] + 2
         e1.record(stream)
         torch.cuda.synchronize()
@@ -462,8 +462,7 @@ def main():
     value = job_rate(ws, npix, ms_max / 1e3)
 
     # per-kernel roofline of the dominant kernel (measured live with CUDA events in the library).
-    # In the overlapped launch shapes the geodesic shares the SMs with the transfers, so its
-    # durations include that sharing; the kernel alone (one pass of each kernel, the shape used
+    # Where transfers run beside the geodesic its durations include that sharing; the kernel alone (one pass of each kernel, the shape used
     # below 2^19 rays) is timed once after the timed region.
     geo_ms, xf_ms = statistics.mean(kt_geo), statistics.mean(kt_xf)
     steps_per_launch = counters["steps"]
@@ -472,8 +471,10 @@ def main():
     shape_note = {0: "one launch per image",
                   1: "overlapped in two workspace halves: each geodesic launch shares the SMs with the "
                      "transfer of the previous chunk",
-                  2: "streamed: one geodesic launch per image beside the transfers of its completed chunks "
-                     f"({counters['transfer_launches']} transfer launches)"}[counters["shape"]]
+                  2: "streamed: one geodesic launch per piece of the image, "
+                     + ("each followed by its transfer" if counters["transfer_launches"] <= geo_launches else
+                        f"beside the transfers of its completed chunks ({counters['transfer_launches']} launches)")
+                  }[counters["shape"]]
     polrt.rt_set_render_config(ctx, 0, 0, 1)
     step()
     alone = polrt.rt_last_counters(ctx)

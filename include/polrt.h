@@ -311,8 +311,9 @@ int rt_image_visibilities(rt_ctx *ctx, const void *img, int form, int stokes, vo
 /* Launch shape of rt_render and rt_render_depths (forms RT_FP64, RT_MIXED, RT_UNPOL).
  * geo_blocks_per_sm and xfer_blocks_per_sm are the resident blocks per SM the geodesic and
  * transfer kernels are launched with (the grid is that times the SM count; 0 = automatic).
- * chunks >= 2 overlaps the two phases, so that the FP64 geodesic and the FP32 transfer share
- * the SMs, in one of two shapes:
+ * chunks >= 2 overlaps the two phases, so that the geodesic and the transfer share the SMs (on
+ * GB300 slower than one after the other: both live on the integer and FP32 pipes), in one of two
+ * shapes:
  *   - streamed, in pieces of the rays that the workspace holds at once (1 when it holds every
  *     ray's path; up to 64; a library-owned workspace first grows to what 60% of the free
  *     device memory allows). The longest-first order is dealt to the pieces, and each piece's
@@ -333,11 +334,12 @@ int rt_image_visibilities(rt_ctx *ctx, const void *img, int form, int stokes, vo
  * chunks 1 runs the phases one after the other on the context's stream.
  * chunks 0 (the default, with {0, 0, 0, 0}) is automatic: RT_MIXED and RT_UNPOL images of 2^19
  * rays or more are overlapped, streamed in chunks of about 2^15 rays (at least 16 per piece)
- * with the geodesic at its full occupancy, or in halves of 4 to 16 chunks of about 2^17 rays with
+ * with the geodesic at its full occupancy (each piece's transfer then follows its geodesic), or in
+ * halves of 4 to 16 chunks of about 2^17 rays with
  * the geodesic at 1 block per SM; smaller images, and the RT_FP64 and RT_SURROGATE forms, run
  * one pass of each kernel. RT_SURROGATE overlaps when chunks >= 2 is set: streamed, each
  * transfer launch's rays go through the features pass, the network (over compact rows) and
- * the transfer in turn; in halves, per chunk (both measured slower than one pass on GB300).
+ * the transfer in turn; in halves, per chunk (no faster than one pass on GB300).
  * Independently of the shape, a full render of 2^17 rays or more (RT_FP64: 2^13) records each
  * pixel's step count, and the next render of the same camera and integrator takes its rays
  * longest first, so that no launch ends waiting for a few long photon-ring rays (smaller images

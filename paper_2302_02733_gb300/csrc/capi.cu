@@ -27,11 +27,14 @@ constexpr int kAutoLastDiv = 1;
 // automatic streamed shape: about 2^kStreamChunkShift rays per chunk, at least 16 per piece, the
 // geodesic at its own occupancy
 constexpr int kStreamChunkShift = 15;
-// Images of fewer rays in one part run in pixel order: they fill the lanes at most about twice, and a warp of
-// only long rays takes longer a step than one whose lanes are leaving (geodesics, pixel order
-// against longest first: 64^2 5.4 / 6.3 ms, 128^2 6.4 / 7.3, 300^2 15.7 / 19, 512^2 25 / 25). The
-// FP64 transfer is bound by its pipe and gains earlier from warps of like lengths (64^2 62.8 / 64 ms,
-// 126 x 130 80 / 72, 300^2 230 / 185).
+// Images of fewer rays in one part run in pixel order. Their lanes are filled about twice at most, and the
+// better order depends on the view: a warp of only long rays takes longer a step than one whose lanes are
+// leaving, and a long ray begun late is waited for. Time in pixel order over longest first, a torus seen
+// from 10 to 160 degrees (mean): mixed 64^2 0.89 to 1.08 (1.00), 128^2 0.86 to 1.01 (0.94), 300^2 0.86 to 1.05
+// (0.96), 362^2 0.99 to 1.17 (1.08), 430^2 1.02 to 1.21 (1.10); FP64 64^2 0.92 to 1.21 (1.07), 126 x 130 0.94
+// to 1.25 (1.08), 200^2 0.84 to 1.07 (0.95), 256^2 0.90 to 1.01 (0.96), 300^2 0.98 to 1.07 (1.02); FP64 ADAF 91 x
+// 90 0.85, 126 x 130 0.95, 200^2 0.94, 300^2 1.00. The mixed line is where the mean crosses 1; in FP64, where it
+// stays within 8% of 1, longest first from 2^13 rays is for the small edge-on images, which gain most.
 constexpr long long kOrderMinRays = 1ll << 17, kOrderMinRaysFp64 = 1ll << 13;
 // RT_FETCH_AUTO: the grid fetch measured faster on GB300 for the benchmark image
 constexpr bool kStagedByDefault = false;
@@ -801,7 +804,7 @@ static int render_streamed(rt_ctx *c, int form, int coef, const Camera &cam, con
         // fits beside the geodesic, or at the transfer's own once the geodesic has ended. Where
         // none fits (the automatic shape), one transfer of the whole piece follows the geodesic:
         // both kernels live on the integer and FP32 pipes, and beside each other they take longer
-        // (1024^2: 79 + 69 ms one after the other; 164 ms at 2 + 2 and 203 ms at 3 + 1 blocks). At
+        // (1024^2: 82 + 61 ms one after the other; 186 ms with 2 geodesic blocks, 219 with 1). At
         // most one launch waits behind the running one: a new launch is made once the previous
         // has started, so the chunks that complete meanwhile join one launch instead of queueing
         // one each (a launch lasts at least as long as its longest ray's transfer).
@@ -1020,12 +1023,13 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     const size_t per_ray = kPerRayBytes + (sur ? (size_t)kBudgetBlocksPerRay * kBlockStates * 48 : 0);
 
     // launch shape: the configured one, or automatic. RT_MIXED and RT_UNPOL overlap images of
-    // 2^19 rays or more: streamed (chunks of about 2^15 rays, the geodesic at its own occupancy)
-    // when the workspace holds a piece of at least 1/64 of the rays, else in two workspace
-    // halves (4 to 16 chunks of about 2^17 rays, the geodesic at 1 block per SM beside the
-    // transfer). Smaller images run one pass of each kernel, and so do RT_FP64 (its FP64
-    // transfer competes with the geodesic for the same pipe) and RT_SURROGATE (the network pass
-    // beside the geodesic measured slower than one pass: 859 against 536 ms).
+    // 2^19 rays or more: streamed (chunks of about 2^15 rays, the geodesic at its own occupancy,
+    // which leaves the transfer no room: it follows) when the workspace holds a piece of at least
+    // 1/64 of the rays, else in two workspace halves (4 to 16 chunks of about 2^17 rays, the
+    // geodesic at 1 block per SM beside the transfer). Smaller images run one pass of each kernel,
+    // and so do RT_FP64 (overlapped transfers are the one-lane kernel: 300^2 121 ms in one pass, 150
+    // overlapped, 600^2 431 and 496) and RT_SURROGATE (1024^2 226 ms either way, 259 with the
+    // network and transfer beside the geodesic).
     int chunks = c->rcfg.chunks, geo_b = c->rcfg.geo_blocks_per_sm, W = c->rcfg.last_chunk_div;
     const bool auto_shape = chunks == 0;
     if (auto_shape)
@@ -1041,7 +1045,7 @@ static int render_impl(rt_ctx *c, int form, void *out_iquv, uint8_t *status, voi
     ChunkLayout L{nrays, 1, 1};
     if (streamed) {
         // contiguous ranges of each piece's longest-first order; the automatic shape takes finer
-        // chunks and a second geodesic block per SM
+        // chunks
         Kp = stream_chunks(nrays, P, chunks, auto_shape);
         if (geo_b == 0) geo_b = c->geo_bps;
     } else {

@@ -28,11 +28,13 @@ __device__ __forceinline__ void therm_eval(const double *t, double u, double &a,
 // A fit converges as rho^-(D + 1), with rho from the distance to the function's nearest singular point in
 // halves of a segment. The Bessel ratios and the logarithm have none nearer than 32 of them (rho 64).
 // f's switch 1 - 1/((X/120)^20 + 1) has poles at 120 exp(+-i pi/20), 18.8 off the real line: with 16
-// segments an octave rho is 19 below X = 128 and 12 from there, which left 1.5e-14 and 4e-12 of f's terms
-// in the octaves beside it; with 64 segments there, 0.8e-15, as evaluated directly. From 256 on they are
-// far enough (1.1e-15).
+// segments an octave rho is 19 below X = 128 and 12 from there, which left 1.5e-14 and 1.6e-12 of f's
+// terms in the octaves beside it; with 64 segments there, 0.8e-15, as evaluated directly. From 256 on they
+// are far enough (1.1e-15).
 // 17 and 19 FP64 instructions in place of 27 reciprocal square roots (14 series terms at z < 2) and of
-// 11 transcendental functions; the FP64 pipe bounds the kernels that read them.
+// 11 transcendental functions; the FP64 pipe bounds the kernels that read them. With fmks_y64 the FP64
+// instructions of 32 states went from 1,721 to 1,343 and the points of a torus at 200^2 from 51 to 36 ms; an
+// ADAF's transfer at 64^2 from 16.4 to 9.5 ms.
 struct ThermTab {
     static constexpr int db = 8, ds = 9;                                  // degrees
     static constexpr int eb = -40, nb = 60 * 16, es = -30, ns = 44 * 16;  // first octave, segments
