@@ -260,7 +260,7 @@ __device__ __forceinline__ unsigned fx_beyond(fx64 m, fx64 lo, fx64 hi) {
 // Every term in 1 / sin is written with P. A negative number in bad is a bound that failed.
 __device__ __forceinline__ void fx_rates(const FxScale &S, const FxState &y, Fx<62> s, Fx<62> c, fx64 nk[4], unsigned &bad) {
     // counts of 64 and more (r above 2^22) leave a sign, as 63 does
-    const int e1 = S.e - 1, g = S.g, g2 = g < 31 ? 2 * g : 63, g3 = g < 21 ? 3 * g : 63;
+    const int e1 = S.e - 1, g = S.g, g2 = 2 * g < 63 ? 2 * g : 63, g3 = 3 * g < 63 ? 3 * g : 63;
     // position terms
     const Fx<64> nal2 = S.nal2.over(g2);
     const Fx<60> na2s2 = nal2 * (s * s);                              // >= -1/4

@@ -31,8 +31,8 @@
 // It is bound by the FP64 pipe, at about 100 instructions a node that emits and 50 one that does not.
 // 8-point Gauss-Legendre panels (16 nodes per unit of s tabulated, 64 exact) with kernels from an
 // interpolated table of logarithms (1.6e-8), or in the exact grade summed at every node, took 51.7 ms
-// for 60,000 points (now 5.5) and 1.1 to 1.6 s for a 64^2 image (now 14 ms of transfer, with its points
-// spread over all lanes), and 58 s for a 20^2 FP64 image (now 13 ms).
+// for 60,000 points (now 5.7 to 6.0) and 1.1 to 1.6 s for a 64^2 image (now 14 ms of transfer, with its
+// points spread over all lanes), and 58 s for a 20^2 FP64 image (now 11 ms of transfer).
 #pragma once
 #include "rt_common.cuh"
 

@@ -8,9 +8,10 @@
 // of screen from one emitting point to the next depend on the geometry alone. So the transfer is
 // two kernels: points_kernel, one warp per ray and one lane per saved state, 32 at a time, replaces
 // each state by its step's record (XRec); chain_kernel, one lane per ray, applies the records in
-// turn. transfer_kernel, one lane per ray for both, runs where the FP64 records have no room. Against it
-// (geodesic excluded): 64^2 mixed 5.8 -> 1.4 ms, 300^2 12 -> 6.0, 1024^2 69 -> 61, and in FP64
-// 64^2 ADAF 63 -> 16 ms, 126 x 130 torus 72 -> 31, 300^2 184 -> 141.
+// turn. transfer_kernel, one lane per ray for both, runs where the FP64 records have no room. Transfers
+// with it and with the two kernels: FP64 ADAF 64^2 39.5 and 9.5 ms, torus 126 x 130 59 and 23, 200^2 85 and
+// 50, 300^2 132 and 104, kappa 20^2 223 and 11; mixed torus 64^2 5.8 and 1.5, 300^2 12 and 6.0, 1024^2 69 and
+// 61.
 #pragma once
 #include <cuda.h>
 
